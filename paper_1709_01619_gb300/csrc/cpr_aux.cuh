@@ -31,25 +31,6 @@ struct AuxArgs {
     double gamma64, ax64, ay64;
 };
 
-// Unsigned division by an invariant divisor d (Granlund & Montgomery,
-// "Division by Invariant Integers using Multiplication", 1994): with
-// l = ceil(log2 d) and m = floor(2^32 (2^l - d) / d) + 1, n / d is
-// (t + ((n - t) >> 1)) >> (l - 1), t the high word of m n, for every 32-bit
-// n; d = 1 is n itself.  div_magic runs on the host.
-inline void div_magic(unsigned int d, unsigned int* m, int* l)
-{
-    int s = 0;
-    while (s < 32 && (1ull << s) < d) ++s;
-    *l = s;
-    *m = (unsigned int)((((1ull << 32) * ((1ull << s) - d)) / d + 1) & 0xffffffffull);
-}
-__device__ __forceinline__ unsigned int div_invariant(unsigned int n, unsigned int d, unsigned int m, int l)
-{
-    if (d == 1u) return n;
-    const unsigned int t = __umulhi(m, n);
-    return (t + ((n - t) >> 1)) >> (l - 1);
-}
-
 // Element average with the same operation order as the stage kernel: row sums
 // with the per-row weights, then the sum over rows.
 template <int N, int V, class T>

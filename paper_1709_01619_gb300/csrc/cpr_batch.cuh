@@ -35,6 +35,8 @@ struct BatchInst {
     long long npts;
     int nx, ny, bcx, bcy;
     int tiles_x, ntiles, tile0;  // tiles of this instance, its first work item
+    unsigned int tx_magic;       // division by tiles_x (div_invariant)
+    int tx_shift;
     T rhx2, rhy2;
     Phys<T> ph;
 };
@@ -48,6 +50,7 @@ struct BatchArgs {
     int swap;          // increment form: the high part of q^n is in Y (else X)
     Tab<T> tab;        // operator tables of the group's order
     TabPr<T> tp;       // the same in pairs over points
+    QuadArgs<T> qx;    // the tables of the quad form (FP32 Euler)
 };
 
 // Register budget: as the single-problem kernel.
@@ -74,6 +77,10 @@ __device__ __forceinline__ void batch_item(const BatchArgs<T>& B, int w, StageAr
         A.bcx = I.bcx;
         A.bcy = I.bcy;
         A.tiles_x = I.tiles_x;
+        if constexpr (sizeof(T) == 4) {
+            A.qx.tx_magic = I.tx_magic;
+            A.qx.tx_shift = I.tx_shift;
+        }
         A.mode = B.mode;
         A.do_avg = 0;
         A.avg = nullptr;
@@ -100,7 +107,10 @@ __device__ __forceinline__ void batch_item(const BatchArgs<T>& B, int w, StageAr
         s_n = I.ntiles;
     }
     __syncthreads();
-    stage_tile<T, P, EQ, DIV, FLUX, TX, TY, DELTA>(sA, B.tab, B.tp, s_t, threadIdx.x, smem_raw, s_n);
+    if constexpr (stage_quad<T, EQ, DELTA>)
+        stage_tile_quad<P, DIV, FLUX, TX, TY, false, 0>(sA, B.tab, B.qx, s_t, threadIdx.x, smem_raw, s_n);
+    else
+        stage_tile<T, P, EQ, DIV, FLUX, TX, TY, DELTA>(sA, B.tab, B.tp, s_t, threadIdx.x, smem_raw, s_n);
 }
 
 // PERSIST: CTAs walk the work list with a grid stride; otherwise the grid

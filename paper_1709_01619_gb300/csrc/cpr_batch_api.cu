@@ -142,6 +142,7 @@ cudaError_t batch_launch(cpr_batch* b, Group& g, int fam, int grid, int mode, in
     B.swap = swap;
     B.tab = cpr::host_tab<T>(b->lcs[g.members[0]].tab);
     B.tp = cpr::host_tabpr<T>(b->lcs[g.members[0]].tab);
+    if constexpr (sizeof(T) == 4) B.qx.tab = cpr::host_quadtab(b->lcs[g.members[0]].tab);
     const LaunchCfg& lc = b->lcs[g.members[0]];
     return fam == 0 ? cpr::batch_fam<T, 0>(g.p, lc.eqn, lc.flux, B, grid, s, 0, nullptr)
                     : cpr::batch_fam<T, 1>(g.p, lc.eqn, lc.flux, B, grid, s, 0, nullptr);
@@ -343,6 +344,7 @@ void fill_tables(cpr_batch* b, Group& g, const void* const* x)
             I.bcx = lc.bcx;
             I.bcy = lc.bcy;
             I.tiles_x = (lc.nx + tx - 1) / tx;
+            cpr::div_magic((unsigned)I.tiles_x, &I.tx_magic, &I.tx_shift);
             I.ntiles = I.tiles_x * ((lc.ny + ty - 1) / ty);
             I.tile0 = tile0;
             tile0 += I.ntiles;
@@ -494,6 +496,7 @@ extern "C" cpr_status cpr_batch_init(const cpr_config* cfgs, int n, void* stream
         // any instances can share (the two-CTA instantiation in per-instance
         // chains measured slower on 64 ragged instances)
         lc.sms = 0;
+        lc.shared = true;
         b->nstate[i] = lc.npts * b->V;
         const size_t bytes = (size_t)b->nstate[i] * esize;
         e = cudaMalloc(&b->Y[i], bytes);

@@ -10,12 +10,12 @@ namespace cpr {
 template <class T, int P, int EQ, int FLUX, int FAM>
 static cudaError_t batch_one(const BatchArgs<T>& B, int grid, cudaStream_t s, int what, int* occ)
 {
-    constexpr int N = P + 1, V = NVars<EQ>::value;
+    constexpr int N = P + 1;
     constexpr int TX = BatchTile<FAM>::X, TY = BatchTile<FAM>::Y;
     constexpr int NT = TX * TY * N;
     auto loop = cpr_batch_stage_kernel<T, P, EQ, DIV_LP, FLUX, TX, TY, stage_delta<T>(), true>;
     auto flat = cpr_batch_stage_kernel<T, P, EQ, DIV_LP, FLUX, TX, TY, stage_delta<T>(), false>;
-    const size_t smem = sizeof(T) * StageLayout<N, V, TX, TY, stage_delta<T>()>::TOTAL;
+    const size_t smem = stage_smem<T, P, EQ, TX, TY, stage_delta<T>()>();
     if (what == 1) {
         cudaError_t e = cudaFuncSetAttribute(loop, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;

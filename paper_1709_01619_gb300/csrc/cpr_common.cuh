@@ -86,13 +86,42 @@ __device__ __forceinline__ float fsqrt(float x)
     return x >= 0.0f ? x * rsqrtf(fmaxf(x, 1.17549435e-38f)) : __int_as_float(0x7fffffff);
 }
 __device__ __forceinline__ double fsqrt(double x) { return sqrt(x); }
+// The same as single instructions (1 ulp and 2^-23; flush-to-zero forms, which
+// leave out the scaling of subnormal operands), for the stage updates (FTZ in
+// the physics below).  The stand-alone FP32 residual keeps the forms above:
+// its relative rounding is that of O(1) fluxes over a small result, so any
+// other rounding would show in it.
+__device__ __forceinline__ float frcp_ftz(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float fsqrt_ftz(float x)
+{
+    float r;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+template <bool FTZ, class T>
+__device__ __forceinline__ T rcp_of(T x)
+{
+    if constexpr (FTZ && sizeof(T) == 4) return frcp_ftz(x);
+    else return frcp(x);
+}
+template <bool FTZ, class T>
+__device__ __forceinline__ T sqrt_of(T x)
+{
+    if constexpr (FTZ && sizeof(T) == 4) return fsqrt_ftz(x);
+    else return fsqrt(x);
+}
 
 // Pressure, Eq. 5: p = (gamma - 1)(e - (rho u u + rho v v)/2) with u = rho u / rho.
 // Also returns r = 1 / rho.
-template <class T>
+template <bool FTZ = false, class T>
 __device__ __forceinline__ T pressure(const T* q, T gamma, T& u, T& v, T& r)
 {
-    r = frcp(q[0]);
+    r = rcp_of<FTZ>(q[0]);
     u = q[1] * r;
     v = q[2] * r;
     return (gamma - T(1)) * (q[3] - T(0.5) * (q[1] * u + q[2] * v));
@@ -137,14 +166,14 @@ __device__ __forceinline__ void flux_y(const T* q, const Phys<T>& ph, T* g)
 
 // Directional derivative of the x- or y-flux, A(q) dq (the chain-rule
 // divergence of Sec. 2.2).  DIR 0: x, 1: y.
-template <int EQ, int DIR, class T>
+template <int EQ, int DIR, bool FTZ = false, class T>
 __device__ __forceinline__ void flux_jvp(const T* q, const T* dq, const Phys<T>& ph, T* df)
 {
     if constexpr (EQ == EQ_ADV) {
         df[0] = (DIR == 0 ? ph.ax : ph.ay) * dq[0];
     } else {
         T u, v, r;
-        T p = pressure(q, ph.gamma, u, v, r);
+        T p = pressure<FTZ>(q, ph.gamma, u, v, r);
         T vn = DIR == 0 ? u : v;
         T dvn = ((DIR == 0 ? dq[1] : dq[2]) - vn * dq[0]) * r;
         T dp = (ph.gamma - T(1)) * (dq[3] - (u * dq[1] + v * dq[2]) + T(0.5) * (u * u + v * v) * dq[0]);
@@ -158,14 +187,16 @@ __device__ __forceinline__ void flux_jvp(const T* q, const T* dq, const Phys<T>&
 // |lambda| of an acoustic field with the Harten-Hyman entropy fix: lam_m,
 // lam_p are the field's speeds at the two states; only across a transonic
 // rarefaction (delta > 0) is |lambda| < delta smoothed.
-template <class T>
+template <bool FTZ, class T>
 __device__ __forceinline__ T roe_abs(T lam, T lam_m, T lam_p)
 {
     T d = T(0);
     d = lam - lam_m > d ? lam - lam_m : d;
     d = lam_p - lam > d ? lam_p - lam : d;
     const T a = lam >= T(0) ? lam : -lam;
-    return a < d ? (lam * lam + d * d) * frcp(T(2) * d) : a;
+    // (FTZ: no 0 / 0 from a subnormal d)
+    const T d2 = FTZ ? ::fmax(T(2) * d, T(1.17549435e-38)) : T(2) * d;
+    return a < d ? (lam * lam + d * d) * rcp_of<FTZ>(d2) : a;
 }
 
 // Roe's flux for the Euler equations through an x-face (DIR 0) or y-face
@@ -173,12 +204,12 @@ __device__ __forceinline__ T roe_abs(T lam, T lam_m, T lam_p)
 // acoustic, entropy and shear fields of the Roe-averaged state (density
 // sqrt(rho_m rho_p); velocity and total enthalpy averaged with weights
 // sqrt(rho)), with the Harten-Hyman fix on the acoustic fields.
-template <int DIR, class T>
+template <int DIR, bool FTZ = false, class T>
 __device__ __forceinline__ void roe_flux(const T* qm, const T* qp, const Phys<T>& ph, T* F)
 {
     const T g = ph.gamma;
     T um, vm, rm, up, vp, rp;
-    const T pm = pressure(qm, g, um, vm, rm), pp = pressure(qp, g, up, vp, rp);
+    const T pm = pressure<FTZ>(qm, g, um, vm, rm), pp = pressure<FTZ>(qp, g, up, vp, rp);
     const T vnm = DIR == 0 ? um : vm, vnp = DIR == 0 ? up : vp;
     T Fm[4], Fp[4];
     Fm[0] = qm[0] * vnm;
@@ -190,11 +221,11 @@ __device__ __forceinline__ void roe_flux(const T* qm, const T* qp, const Phys<T>
     Fm[3] = (qm[3] + pm) * vnm;
     Fp[3] = (qp[3] + pp) * vnp;
     const T Hm = (qm[3] + pm) * rm, Hp = (qp[3] + pp) * rp;
-    const T wm = fsqrt(qm[0]), wp = fsqrt(qp[0]), iw = frcp(wm + wp);
+    const T wm = sqrt_of<FTZ>(qm[0]), wp = sqrt_of<FTZ>(qp[0]), iw = rcp_of<FTZ>(wm + wp);
     const T rho = wm * wp;
     const T u = (wm * um + wp * up) * iw, v = (wm * vm + wp * vp) * iw, H = (wm * Hm + wp * Hp) * iw;
     const T c2 = (g - T(1)) * (H - T(0.5) * (u * u + v * v));
-    const T cs = fsqrt(c2), ic2 = frcp(c2);
+    const T cs = sqrt_of<FTZ>(c2), ic2 = rcp_of<FTZ>(c2);
     const T vn = DIR == 0 ? u : v;
     const T vt = DIR == 0 ? v : -u;  // along t = (-n_y, n_x)
     const T dvn = vnp - vnm;
@@ -204,10 +235,10 @@ __device__ __forceinline__ void roe_flux(const T* qm, const T* qp, const Phys<T>
     const T a2 = (qp[0] - qm[0]) - dp * ic2;
     const T a3 = rho * dvt;
     const T a4 = (dp + rho * cs * dvn) * T(0.5) * ic2;
-    const T cm = fsqrt(g * pm * rm), cp = fsqrt(g * pp * rp);
-    const T l1 = roe_abs(vn - cs, vnm - cm, vnp - cp);
+    const T cm = sqrt_of<FTZ>(g * pm * rm), cp = sqrt_of<FTZ>(g * pp * rp);
+    const T l1 = roe_abs<FTZ>(vn - cs, vnm - cm, vnp - cp);
     const T l2 = vn >= T(0) ? vn : -vn;
-    const T l4 = roe_abs(vn + cs, vnm + cm, vnp + cp);
+    const T l4 = roe_abs<FTZ>(vn + cs, vnm + cm, vnp + cp);
     const T nx = DIR == 0 ? T(1) : T(0), ny = DIR == 0 ? T(0) : T(1);
     const T r1[4] = {T(1), u - cs * nx, v - cs * ny, H - vn * cs};
     const T r2[4] = {T(1), u, v, T(0.5) * (u * u + v * v)};
@@ -263,15 +294,15 @@ __device__ __forceinline__ void common_flux(const T* qm, const T* qp, const Phys
 }
 
 // Largest signal speed sqrt(u^2 + v^2) + c at one point (Eq. 36).
-template <int EQ, class T>
+template <int EQ, bool FTZ = false, class T>
 __device__ __forceinline__ T point_speed(const T* q, const Phys<T>& ph)
 {
     if constexpr (EQ == EQ_ADV) {
         return fsqrt(ph.ax * ph.ax + ph.ay * ph.ay);
     } else {
         T u, v, r;
-        T p = pressure(q, ph.gamma, u, v, r);
-        return fsqrt(u * u + v * v) + fsqrt(ph.gamma * p * r);
+        T p = pressure<FTZ>(q, ph.gamma, u, v, r);
+        return sqrt_of<FTZ>(u * u + v * v) + sqrt_of<FTZ>(ph.gamma * p * r);
     }
 }
 
@@ -599,5 +630,36 @@ struct TabPr {
     Pr<T> lm2[(kMaxN + 1) / 2], lp2[(kMaxN + 1) / 2];
     Pr<T> dgl2[(kMaxN + 1) / 2], dgr2[(kMaxN + 1) / 2];
 };
+
+// Operator tables of the quad form (cpr_stage_quad.cuh), which uses the
+// symmetry of the solution points: lm[l] = l_l(-1) = l_{N-1-l}(+1); dgl[a] =
+// g_L'(xi_a) = -g_R'(xi_{N-1-a}); and the derivative as a combination of the
+// N - 1 differences f_{m+1} - f_m, f'_a = sum_m C_am (f_{m+1} - f_m), with C_am
+// = sum_{l > m} D_al = C_{N-1-a,N-2-m}, split over mirrored differences:
+// ce = (C_am + C_a,N-2-m) / 2, co = (C_am - C_a,N-2-m) / 2, cm the middle
+// difference's (even N).
+struct QuadTab {
+    float lm[kMaxN], dgl[kMaxN];
+    float ce[(kMaxN + 1) / 2][2], co[(kMaxN + 1) / 2][2], cm[(kMaxN + 1) / 2];
+};
+
+// Unsigned division by an invariant divisor d (Granlund & Montgomery,
+// "Division by Invariant Integers using Multiplication", 1994): with
+// l = ceil(log2 d) and m = floor(2^32 (2^l - d) / d) + 1, n / d is
+// (t + ((n - t) >> 1)) >> (l - 1), t the high word of m n, for every 32-bit
+// n; d = 1 is n itself.  div_magic runs on the host.
+inline void div_magic(unsigned int d, unsigned int* m, int* l)
+{
+    int s = 0;
+    while (s < 32 && (1ull << s) < d) ++s;
+    *l = s;
+    *m = (unsigned int)((((1ull << 32) * ((1ull << s) - d)) / d + 1) & 0xffffffffull);
+}
+__device__ __forceinline__ unsigned int div_invariant(unsigned int n, unsigned int d, unsigned int m, int l)
+{
+    if (d == 1u) return n;
+    const unsigned int t = __umulhi(m, n);
+    return (t + ((n - t) >> 1)) >> (l - 1);
+}
 
 }  // namespace cpr

@@ -29,6 +29,7 @@ struct LaunchCfg {
     long long l2_bytes;     // L2 size of the device (0: unknown)
     int sms;                // SMs of the device: a stage launch of at most two CTAs per SM takes
                             // the instantiation compiled for two resident CTAs (0: never)
+    bool shared;            // an instance of a batch: its launches share the SMs with other instances
     int nx, ny, bcx, bcy;
     long long ne, npts;
     double hx, hy, gamma, ax, ay, tvb_M, lim_eps;

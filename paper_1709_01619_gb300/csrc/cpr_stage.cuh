@@ -48,6 +48,17 @@
 
 namespace cpr {
 
+// What only the quad form (FP32 Euler) needs: its tables and the division of
+// a tile index by tiles_x (div_invariant).  Nothing for FP64.
+template <class T>
+struct QuadArgs {};
+template <>
+struct QuadArgs<float> {
+    QuadTab tab;
+    unsigned int tx_magic;
+    int tx_shift;
+};
+
 template <class T>
 struct StageArgs {
     const T* qs;      // stage input state (increment modes: hi of q^n)
@@ -68,6 +79,7 @@ struct StageArgs {
     Phys<T> ph;
     Tab<T> tab;
     TabPr<T> tp;      // the tables in pairs over points (two-lane path)
+    QuadArgs<T> qx;   // the quad form's own arguments (FP32 Euler)
 };
 
 template <int N, int V, int TX, int TY, bool DELTA>
@@ -351,6 +363,25 @@ constexpr int stage_min_blocks()
                            : (N == 2 ? CPR_STAGE_MINB_FP32_N2
                                      : (N == 3 ? CPR_STAGE_MINB_FP32_N3
                                                : (N == 4 ? CPR_STAGE_MINB_FP32 : CPR_STAGE_MINB_FP32_N5))));
+}
+
+}  // namespace cpr
+
+#include "cpr_stage_quad.cuh"
+
+namespace cpr {
+
+// The FP32 Euler stage updates take the quad form (the stand-alone residual
+// the one below).
+template <class T, int EQ, bool DELTA>
+constexpr bool stage_quad = sizeof(T) == 4 && EQ == EQ_EULER && !DELTA;
+
+// Dynamic shared memory of a stage-update CTA.
+template <class T, int P, int EQ, int TX, int TY, bool DELTA>
+constexpr size_t stage_smem()
+{
+    if constexpr (stage_quad<T, EQ, DELTA>) return sizeof(Quad) * QuadLayout<P + 1, TX, TY>::TOTAL;
+    else return sizeof(T) * StageLayout<P + 1, NVars<EQ>::value, TX, TY, DELTA>::TOTAL;
 }
 
 // One tile of the stage: the work of one CTA.  tile indexes the instance's
@@ -906,13 +937,19 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, const Tab<T>& 
 // PF: the instantiation for compensated stages whose states exceed L2 (it
 // prefetches the low part; launched only when StageArgs::pf_lo is set).
 template <class T, int P, int EQ, int DIV, int FLUX, int TX, int TY, bool DELTA, bool PF = false, bool WIDE = false>
-__global__ void __launch_bounds__(TX * TY * (P + 1), (stage_min_blocks<T, P + 1, WIDE, TX * TY>()))
+__global__ void __launch_bounds__(TX * TY * (P + 1),
+                                  (PF && stage_quad<T, EQ, DELTA> ? quad_min_blocks<P, WIDE, TX * TY>()
+                                                                  : stage_min_blocks<T, P + 1, WIDE, TX * TY>()))
 cpr_stage_kernel(const StageArgs<T> A)
 {
     static_assert((TX * TY * (P + 1)) % 32 == 0, "whole warps: the warp-level reductions use every lane");
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    stage_tile<T, P, EQ, DIV, FLUX, TX, TY, DELTA, PF>(A, A.tab, A.tp, blockIdx.x, threadIdx.x, smem_raw,
-                                                       gridDim.x);
+    if constexpr (PF && stage_quad<T, EQ, DELTA>)
+        stage_tile_quad<P, DIV, FLUX, TX, TY, true, MODE_INC3>(A, A.tab, A.qx, blockIdx.x, threadIdx.x, smem_raw,
+                                                              gridDim.x);
+    else
+        stage_tile<T, P, EQ, DIV, FLUX, TX, TY, DELTA, PF>(A, A.tab, A.tp, blockIdx.x, threadIdx.x, smem_raw,
+                                                           gridDim.x);
 }
 
 }  // namespace cpr

@@ -3,6 +3,8 @@
 // in parallel.
 #pragma once
 
+#include <type_traits>
+
 #include "cpr_launch.h"
 #include "cpr_tabconv.cuh"
 #include "cpr_stage.cuh"
@@ -17,25 +19,65 @@
 namespace cpr {
 
 
+// The FP32 Euler stage updates (quad form).  A single problem with the LP
+// divergence and Rusanov's flux takes a kernel compiled for the stage mode
+// (1-6; the arrays it reads and its update are then fixed at compile time:
+// 1024^2 p = 3 4.63 -> 4.51 ms for 8 steps, 128^2 1.178 -> 1.105 ms for 64);
+// other divergences and fluxes one kernel for every mode.  So does an instance
+// of a batch: its SMs run CTAs of every order and stage at once, and the
+// kernels of three orders and three modes evict one another's instructions
+// (64 instances, 24 steps: 32.5 ms with one kernel per order, 35.0 with three).
+template <int P, int DIV, int FLUX, int TX, int TY, class F>
+static cudaError_t with_quad_kernel(int mode, bool wide, bool shared, F&& f)
+{
+    constexpr int E = TX * TY, MB = quad_min_blocks<P, false, E>(), MW = quad_min_blocks<P, true, E>();
+    constexpr int MS = stage_min_blocks<float, P + 1, false, E>();
+    if (shared) return f(cpr_stage_quad_kernel<P, DIV, FLUX, TX, TY, MS, 0>);
+    if constexpr (DIV == DIV_LP && FLUX == FLUX_RUSANOV) {
+        auto pick = [&](auto m) {
+            constexpr int M = decltype(m)::value;
+            return wide ? f(cpr_stage_quad_kernel<P, DIV, FLUX, TX, TY, MW, M>)
+                        : f(cpr_stage_quad_kernel<P, DIV, FLUX, TX, TY, MB, M>);
+        };
+        switch (mode) {
+        case MODE_SO1: return pick(std::integral_constant<int, MODE_SO1>{});
+        case MODE_SO2: return pick(std::integral_constant<int, MODE_SO2>{});
+        case MODE_SO3: return pick(std::integral_constant<int, MODE_SO3>{});
+        case MODE_INC1: return pick(std::integral_constant<int, MODE_INC1>{});
+        case MODE_INC2: return pick(std::integral_constant<int, MODE_INC2>{});
+        default: return pick(std::integral_constant<int, MODE_INC3>{});
+        }
+    } else {
+        return wide ? f(cpr_stage_quad_kernel<P, DIV, FLUX, TX, TY, MW, 0>)
+                    : f(cpr_stage_quad_kernel<P, DIV, FLUX, TX, TY, MB, 0>);
+    }
+}
+
 template <class T, int P, int EQ, int DIV, int FLUX>
 static cudaError_t stage_one(const LaunchCfg& c, const StageArgs<T>& A, int ctas, cudaStream_t s, bool prep)
 {
     constexpr int N = P + 1, V = NVars<EQ>::value;
     constexpr int TX = stage_tile_x(P), TY = stage_tile_y(P);
     constexpr int NT = TX * TY * N;
-    const size_t smem = sizeof(T) * StageLayout<N, V, TX, TY, stage_delta<T>()>::TOTAL;
-    auto kern = cpr_stage_kernel<T, P, EQ, DIV, FLUX, TX, TY, stage_delta<T>()>;
+    constexpr bool DELTA = stage_delta<T>();
+    // FP32 Euler: the quad form for the stage updates; the stand-alone
+    // residual, and every other type and equation, the general kernel
+    constexpr bool QUAD = stage_quad<T, EQ, DELTA>;
+    const size_t smem = sizeof(T) * StageLayout<N, V, TX, TY, DELTA>::TOTAL;
+    [[maybe_unused]] const size_t smem_q = stage_smem<T, P, EQ, TX, TY, DELTA>();
+    auto kern = cpr_stage_kernel<T, P, EQ, DIV, FLUX, TX, TY, DELTA>;
     // the prefetching instantiation only where the compensated FP32 stages
     // run on large states: Euler, LP divergence, Rusanov flux
     constexpr bool HAS_PF = sizeof(T) == 4 && EQ == EQ_EULER && DIV == DIV_LP && FLUX == FLUX_RUSANOV;
-    auto kern_pf = cpr_stage_kernel<T, P, EQ, DIV, FLUX, TX, TY, stage_delta<T>(), HAS_PF>;
+    auto kern_pf = cpr_stage_kernel<T, P, EQ, DIV, FLUX, TX, TY, DELTA, HAS_PF>;
     // and the one for grids of at most two CTAs per SM: FP32 Euler, every
     // divergence and flux
     constexpr bool HAS_WIDE = sizeof(T) == 4 && EQ == EQ_EULER;
-    auto kern_w = cpr_stage_kernel<T, P, EQ, DIV, FLUX, TX, TY, stage_delta<T>(), false, HAS_WIDE>;
+    auto kern_w = cpr_stage_kernel<T, P, EQ, DIV, FLUX, TX, TY, DELTA, false, HAS_WIDE>;
     // CTAs per SM the wide instantiation is compiled for: the grid fits the
     // device at once up to that many per SM
     constexpr int WIDE_PER_SM = stage_min_blocks<T, N, true, TX * TY>();
+    const bool wide = HAS_WIDE && c.sms > 0 && ctas <= WIDE_PER_SM * c.sms;
     // and, in FP64, tiles of 4 x 4 elements for grids of at most one tile per
     // two SMs: four times the CTAs, so that more SMs share the FP64 work of a
     // grid that would leave most of them idle (Euler, LP divergence, Rusanov
@@ -46,17 +88,23 @@ static cudaError_t stage_one(const LaunchCfg& c, const StageArgs<T>& A, int ctas
     constexpr int SX = 4, SY = 4;
     constexpr bool HAS_SMALL = sizeof(T) == 8 && EQ == EQ_EULER && DIV == DIV_LP && FLUX == FLUX_RUSANOV &&
                                (SX * SY * N) % 32 == 0 && CPR_STAGE_SMALL != 0;
-    [[maybe_unused]] const size_t smem_s = sizeof(T) * StageLayout<N, V, SX, SY, stage_delta<T>()>::TOTAL;
+    [[maybe_unused]] const size_t smem_s = sizeof(T) * StageLayout<N, V, SX, SY, DELTA>::TOTAL;
     if (prep) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e == cudaSuccess && HAS_PF)
-            e = cudaFuncSetAttribute(kern_pf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e == cudaSuccess && HAS_WIDE)
-            e = cudaFuncSetAttribute(kern_w, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        auto limit = [](auto k, size_t bytes) {
+            return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        };
+        cudaError_t e = limit(kern, smem);
+        if (e == cudaSuccess && HAS_PF) e = limit(kern_pf, QUAD ? smem_q : smem);
+        if (e == cudaSuccess && HAS_WIDE) e = limit(kern_w, smem);
         if constexpr (HAS_SMALL)
             if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(cpr_stage_kernel<T, P, EQ, DIV, FLUX, SX, SY, stage_delta<T>(), false, true>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_s);
+                e = limit(cpr_stage_kernel<T, P, EQ, DIV, FLUX, SX, SY, DELTA, false, true>, smem_s);
+        if constexpr (QUAD)
+            for (int mode = MODE_SO1; mode <= MODE_INC3 && e == cudaSuccess; ++mode) {
+                auto lq = [&](auto k) { return limit(k, smem_q); };
+                e = with_quad_kernel<P, DIV, FLUX, TX, TY>(mode, false, c.shared, lq);
+                if (e == cudaSuccess) e = with_quad_kernel<P, DIV, FLUX, TX, TY>(mode, true, c.shared, lq);
+            }
         return e;
     }
     if constexpr (HAS_SMALL) {
@@ -64,13 +112,23 @@ static cudaError_t stage_one(const LaunchCfg& c, const StageArgs<T>& A, int ctas
             StageArgs<T> As = A;
             As.tiles_x = (c.nx + SX - 1) / SX;
             const int grid = As.tiles_x * ((c.ny + SY - 1) / SY);
-            cpr_stage_kernel<T, P, EQ, DIV, FLUX, SX, SY, stage_delta<T>(), false, true>
+            cpr_stage_kernel<T, P, EQ, DIV, FLUX, SX, SY, DELTA, false, true>
                 <<<grid, SX * SY * N, smem_s, s>>>(As);
             return cudaGetLastError();
         }
     }
+    if constexpr (QUAD) {
+        if (A.mode != MODE_RESIDUAL) {
+            auto launch = [&](auto k) {
+                k<<<ctas, NT, smem_q, s>>>(A);
+                return cudaGetLastError();
+            };
+            if (HAS_PF && A.pf_lo && !c.shared) return launch(kern_pf);
+            return with_quad_kernel<P, DIV, FLUX, TX, TY>(A.mode, wide, c.shared, launch);
+        }
+    }
     if (HAS_PF && A.pf_lo) kern_pf<<<ctas, NT, smem, s>>>(A);
-    else if (HAS_WIDE && c.sms > 0 && ctas <= WIDE_PER_SM * c.sms) kern_w<<<ctas, NT, smem, s>>>(A);
+    else if (wide) kern_w<<<ctas, NT, smem, s>>>(A);
     else kern<<<ctas, NT, smem, s>>>(A);
     return cudaGetLastError();
 }
@@ -122,6 +180,10 @@ static StageArgs<T> make_stage_args(const LaunchCfg& c, int mode, const StagePtr
     A.ph.ay = T(c.ay);
     A.tab = host_tab<T>(c.tab);
     A.tp = host_tabpr<T>(c.tab);
+    if constexpr (sizeof(T) == 4) {
+        A.qx.tab = host_quadtab(c.tab);
+        div_magic((unsigned)A.tiles_x, &A.qx.tx_magic, &A.qx.tx_shift);
+    }
     return A;
 }
 

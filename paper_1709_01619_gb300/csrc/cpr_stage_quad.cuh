@@ -1,0 +1,556 @@
+// cpr_stage_quad.cuh -- the tile of the fused residual + SSP-RK3 stage for the
+// FP32 Euler equations (the scheme and its stage modes: cpr_stage.cuh).
+//
+// The four variables of a point are kept together: shared memory holds one
+// 16-byte quad (rho, rho u, rho v, e) per point, edge state, edge flux or
+// jump, so that each of them is one 16-byte access instead of four words, and
+// the line operators run on pairs of variables (packed FP32 instructions)
+// with a table entry broadcast to both lanes: no lane is padding for any
+// order and no sum runs across lanes.
+//
+// Against the same phases with one word per variable (thread instructions per
+// thread of the first increment stage: p = 2 1185 -> 695, p = 3 1080 -> 848,
+// p = 4 1450 -> 961), per pass: 1024^2 p = 3 5.27 -> 4.51 ms (8 steps), 1365 x
+// 1363 p = 2 5.67 -> 4.70 ms (6 steps), 821 x 819 p = 4 5.64 -> 5.03 ms (6
+// steps), 128^2 p = 3 1.34 -> 1.11 ms (64 steps, L2-resident).
+#pragma once
+
+#include "cpr_common.cuh"
+#include "cpr_reduce.cuh"
+
+namespace cpr {
+
+struct alignas(16) Quad {
+    Pr<float> a, b;  // (rho, rho u), (rho v, e)
+};
+
+__device__ __forceinline__ Quad qmk(float x, float y, float z, float w) { return {pmk(x, y), pmk(z, w)}; }
+__device__ __forceinline__ Quad qmul(const Quad& x, float c) { return {pmul(pbc(c), x.a), pmul(pbc(c), x.b)}; }
+__device__ __forceinline__ Quad qfma(const Quad& x, float c, const Quad& y)
+{
+    return {pfma(pbc(c), x.a, y.a), pfma(pbc(c), x.b, y.b)};
+}
+__device__ __forceinline__ Quad qadd(const Quad& x, const Quad& y) { return {padd(x.a, y.a), padd(x.b, y.b)}; }
+__device__ __forceinline__ Quad qsub(const Quad& x, const Quad& y) { return {psub(x.a, y.a), psub(x.b, y.b)}; }
+__device__ __forceinline__ void qget(const Quad& x, float* v)
+{
+    v[0] = x.a.v.x;
+    v[1] = x.a.v.y;
+    v[2] = x.b.v.x;
+    v[3] = x.b.v.y;
+}
+__device__ __forceinline__ Quad qput(const float* v) { return qmk(v[0], v[1], v[2], v[3]); }
+
+// Edge states of a line of N quads at -1 (lo) and +1 (hi).  The solution
+// points are symmetric, so l_l(+1) = l_{N-1-l}(-1): one table serves both.
+// Every edge state of the kernel, the element's own and the one a neighbour
+// CTA forms from its halo line, is one of these two sums in this order.
+template <int N>
+__device__ __forceinline__ Quad edge_lo(const QuadTab& t, const Quad (&x)[N])
+{
+    Quad s = qmul(x[0], t.lm[0]);
+#pragma unroll
+    for (int l = 1; l < N; ++l) s = qfma(x[l], t.lm[l], s);
+    return s;
+}
+template <int N>
+__device__ __forceinline__ Quad edge_hi(const QuadTab& t, const Quad (&x)[N])
+{
+    Quad s = qmul(x[N - 1], t.lm[0]);
+#pragma unroll
+    for (int l = 1; l < N; ++l) s = qfma(x[N - 1 - l], t.lm[l], s);
+    return s;
+}
+
+// Derivative of the interpolant of a line at its N points.  The rows of D sum
+// to zero, so it is a combination of the N - 1 differences of neighbouring
+// values (exact for values within a factor of two, where the plain row sum
+// rounds every product of an O(1) value); and D changes sign under the mirror
+// image of the line, so sums and differences of mirrored differences serve
+// two points at once: 8 / 13 / 22 operations per pair of variables for
+// N = 3 / 4 / 5 against 9 / 16 / 25 of the row sums.
+template <int N>
+__device__ __forceinline__ void line_derivative(const QuadTab& t, const Quad (&f)[N], Quad (&r)[N])
+{
+    constexpr int M = N - 1, H = M / 2;
+    Quad s[H > 0 ? H : 1], d[H > 0 ? H : 1], mid;
+#pragma unroll
+    for (int m = 0; m < H; ++m) {
+        const Quad lo = qsub(f[m + 1], f[m]), hi = qsub(f[N - 1 - m], f[N - 2 - m]);
+        s[m] = qadd(lo, hi);
+        d[m] = qsub(lo, hi);
+    }
+    if constexpr (M % 2 == 1) mid = qsub(f[H + 1], f[H]);
+#pragma unroll
+    for (int a = 0; a < (N + 1) / 2; ++a) {
+        Quad p;
+        if constexpr (M % 2 == 1) {
+            p = qmul(mid, t.cm[a]);
+#pragma unroll
+            for (int m = 0; m < H; ++m) p = qfma(s[m], t.ce[a][m], p);
+        } else {
+            p = qmul(s[0], t.ce[a][0]);
+#pragma unroll
+            for (int m = 1; m < H; ++m) p = qfma(s[m], t.ce[a][m], p);
+        }
+        if (2 * a == N - 1) {
+            r[a] = p;
+        } else {
+            Quad lo = p, hi = p;
+#pragma unroll
+            for (int m = 0; m < H; ++m) {
+                lo = qfma(d[m], t.co[a][m], lo);
+                hi = qfma(d[m], -t.co[a][m], hi);
+            }
+            r[a] = lo;
+            r[N - 1 - a] = hi;
+        }
+    }
+}
+
+// Shared memory of a tile, in quads.
+template <int N, int TX, int TY>
+struct QuadLayout {
+    static constexpr int NN = N * N, E = TX * TY;
+    static constexpr int SQ = E * NN;             // tile copy of the stage input, then the y-part of the residual
+    static constexpr int XR = TY * (TX + 1) * N;  // right edge states, elements -1..TX-1
+    static constexpr int XH = TY * N;             // left edge states of the right halo
+    static constexpr int XF = E * N;              // right edge fluxes, then the right jumps
+    static constexpr int YT = (TY + 1) * TX * N;  // top edge states, elements -1..TY-1
+    static constexpr int YH = TX * N;             // bottom edge states of the upper halo
+    static constexpr int YF = E * N;              // top edge fluxes, then the top jumps
+    static constexpr int TOTAL = SQ + XR + XH + XF + YT + YH + YF;
+    // Point (b, a) of element el.  A quarter warp's accesses (eight threads,
+    // 16 bytes each) must hit distinct 16-byte columns of the 128-byte bank
+    // row, for the rows (thread = row b, one store per a) and for the columns
+    // (thread = column a, one load per b).  N = 4: eight threads hold two
+    // elements; XOR of the row into the column and of the element's parity
+    // into the row.  N = 2: four elements.  N = 3, 5: the odd element stride
+    // does it for the rows, and for the columns when a warp holds one column
+    // of consecutive elements (the k-major identity of phase 2).
+    __device__ static int sq(int el, int b, int a)
+    {
+        if constexpr (N == 4) return el * 16 + ((b ^ (el & 1)) << 2) + (a ^ b);
+        else if constexpr (N == 2) return el * 4 + ((b * 2 + a) ^ (((el >> 1) & 1) * 3));
+        else return el * NN + b * N + a;
+    }
+    __device__ static int xr(int ty, int f, int k) { return (ty * (TX + 1) + f) * N + k; }
+    __device__ static int yt(int g, int tx, int k) { return (g * TX + tx) * N + k; }
+    __device__ static int ef(int el, int k) { return el * N + k; }
+};
+
+// Row of N values of every variable (point offset off) as quads; addb adds
+// the increment array.
+template <int N>
+__device__ __forceinline__ void load_row_quads(const float* __restrict__ q, const float* __restrict__ qb, bool addb,
+                                               long long npts, long long off, Quad (&x)[N])
+{
+    float r[4][N];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) gload_row<N>(q + v * npts + off, r[v]);
+    if (addb) {
+        float b[4][N];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) gload_row<N>(qb + v * npts + off, b[v]);
+#pragma unroll
+        for (int v = 0; v < 4; ++v)
+#pragma unroll
+            for (int a = 0; a < N; ++a) r[v][a] += b[v][a];
+    }
+#pragma unroll
+    for (int a = 0; a < N; ++a) x[a] = qmk(r[0][a], r[1][a], r[2][a], r[3][a]);
+}
+
+// Column of N values (stride N) of every variable as quads.
+template <int N>
+__device__ __forceinline__ void load_col_quads(const float* __restrict__ q, const float* __restrict__ qb, bool addb,
+                                               long long npts, long long off, Quad (&x)[N])
+{
+    float r[4][N];
+#pragma unroll
+    for (int v = 0; v < 4; ++v)
+#pragma unroll
+        for (int l = 0; l < N; ++l) r[v][l] = q[v * npts + off + l * N];
+    if (addb) {
+        float b[4][N];
+#pragma unroll
+        for (int v = 0; v < 4; ++v)
+#pragma unroll
+            for (int l = 0; l < N; ++l) b[v][l] = qb[v * npts + off + l * N];
+#pragma unroll
+        for (int v = 0; v < 4; ++v)
+#pragma unroll
+            for (int l = 0; l < N; ++l) r[v][l] += b[v][l];
+    }
+#pragma unroll
+    for (int a = 0; a < N; ++a) x[a] = qmk(r[0][a], r[1][a], r[2][a], r[3][a]);
+}
+
+// Flux of Eq. 4 through DIR at one point; SPEED: also the signal speed
+// |Vn| + c.
+template <int DIR, bool SPEED = false>
+__device__ __forceinline__ Quad quad_flux(const Quad& q, const Phys<float>& ph, float* s = nullptr)
+{
+    float v[4], u, w, r;
+    qget(q, v);
+    const float p = pressure<true>(v, ph.gamma, u, w, r);
+    const float vn = DIR == 0 ? u : w;
+    if constexpr (SPEED) *s = fabsf(vn) + fsqrt_ftz(ph.gamma * p * r);
+    const float h = (v[3] + p) * vn;
+    if constexpr (DIR == 0) return qmk(v[1], fmaf(v[1], u, p), v[2] * u, h);
+    else return qmk(v[2], v[1] * w, fmaf(v[2], w, p), h);
+}
+
+// Twice the common flux through a face between the lower state m and the
+// upper state p (the factor 1/2 joins the jump's subtraction, half_jump).
+template <int FLUX, int DIR>
+__device__ __forceinline__ Quad quad_face2(const Quad& m, const Quad& p, const Phys<float>& ph)
+{
+    if constexpr (FLUX == FLUX_RUSANOV) {
+        float sm, sp;
+        const Quad fm = quad_flux<DIR, true>(m, ph, &sm), fp = quad_flux<DIR, true>(p, ph, &sp);
+        const float lam = sm >= sp ? sm : sp;
+        return qfma(qsub(m, p), lam, qadd(fm, fp));
+    } else {
+        float a[4], b[4], F[4];
+        qget(m, a);
+        qget(p, b);
+        roe_flux<DIR, true>(a, b, ph, F);
+        return qmul(qput(F), 2.f);
+    }
+}
+// F* - f from twice the common flux.
+__device__ __forceinline__ Quad half_jump(const Quad& G2, const Quad& f)
+{
+    return {pfma(G2.a, pbc(0.5f), pmul(f.a, pbc(-1.f))), pfma(G2.b, pbc(0.5f), pmul(f.b, pbc(-1.f)))};
+}
+
+// x-line or y-line of one thread: derivative r, edge states lo, hi and edge
+// fluxes flo, fhi of the line x (consumed).
+template <int N, int DIR, int DIV>
+__device__ __forceinline__ void quad_line(const QuadTab& t, const Phys<float>& ph, Quad (&x)[N], Quad (&r)[N],
+                                          Quad& lo, Quad& hi, Quad& flo, Quad& fhi)
+{
+    lo = edge_lo<N>(t, x);
+    hi = edge_hi<N>(t, x);
+    if constexpr (DIV == DIV_LP) {
+#pragma unroll
+        for (int a = 0; a < N; ++a) x[a] = quad_flux<DIR>(x[a], ph);
+        flo = edge_lo<N>(t, x);
+        fhi = edge_hi<N>(t, x);
+        line_derivative<N>(t, x, r);
+    } else {
+        Quad dq[N];
+        line_derivative<N>(t, x, dq);
+#pragma unroll
+        for (int a = 0; a < N; ++a) {
+            float q[4], d[4], o[4];
+            qget(x[a], q);
+            qget(dq[a], d);
+            flux_jvp<EQ_EULER, DIR, true>(q, d, ph, o);
+            r[a] = qput(o);
+        }
+        flo = quad_flux<DIR>(lo, ph);
+        fhi = quad_flux<DIR>(hi, ph);
+    }
+}
+
+// One tile of a stage update (modes 1-6): the work of one CTA (the tile
+// index, the idle threads and nslots: stage_tile of cpr_stage.cuh).  MODE: the
+// stage mode, or 0 for the one in the arguments.
+//
+// Thread (el, k) is row k of element el in phases 1 and 4 and a column of an
+// element in phases 2 and 3.
+//   1 halo lines (edge states of the neighbour elements facing the tile, one
+//     line of all variables per thread), own row: into the tile copy, x-line
+//   2 column from the tile copy: y-line
+//   3 common flux on the element's left and lower face points, one evaluation
+//     per face point (the tile's right / upper edge faces go to threads of
+//     their own), and the jumps F* - f of both elements: the neighbour's over
+//     its edge flux, the own lower one into the y-derivative, which goes over
+//     the dead tile copy
+//   4 row k: corrections, stage update, store; averages, CFL maximum
+template <int P, int DIV, int FLUX, int TX, int TY, bool PF, int MODE>
+__device__ __forceinline__ void stage_tile_quad(const StageArgs<float>& A, const Tab<float>& tb, const QuadArgs<float>& qx,
+                                                int tile, int tid, unsigned char* smem_raw, int nslots)
+{
+    constexpr int N = P + 1, NN = N * N;
+    constexpr int NT = TX * TY * N;
+    using L = QuadLayout<N, TX, TY>;
+    Quad* sq = reinterpret_cast<Quad*>(smem_raw);
+    Quad* xR = sq + L::SQ;
+    Quad* xH = xR + L::XR;
+    Quad* xF = xH + L::XH;
+    Quad* yT = xF + L::XF;
+    Quad* yH = yT + L::YT;
+    Quad* yF = yH + L::YH;
+    Quad* avS = xR;  // row partial sums of the averages, over the edge states after phase 3
+    static_assert(L::XR >= TX * TY * N, "the partial sums of the averages fit the right edge states");
+
+    const int mode = MODE > 0 ? MODE : A.mode;
+    if (A.ctrl->done) return;  // t_end reached: uniform exit
+    // a limited run: clear the marked-element count of the limiter pass
+    // that follows this stage (stream order keeps it apart from the last one)
+    if (A.do_avg && tile == 0 && tid == 0) A.ctrl->marked = 0;
+
+    const bool active = tid < NT;
+    const QuadTab& qt = qx.tab;
+    const int tj = (int)div_invariant((unsigned)tile, (unsigned)A.tiles_x, A.qx.tx_magic, A.qx.tx_shift);
+    const int i0 = (tile - tj * A.tiles_x) * TX;
+    const int j0 = tj * TY;
+    const int TXe = min(TX, A.nx - i0), TYe = min(TY, A.ny - j0);
+    const int el = tid / N, k = tid % N;
+    const int tx = el % TX, ty = el / TX;
+    const bool valid = active && tx < TXe && ty < TYe;
+    const long long e = (long long)(j0 + ty) * A.nx + (i0 + tx);
+    const long long off = e * NN + k * N;
+    const bool addb = mode == MODE_INC2 || mode == MODE_INC3;
+    const bool lwall = A.bcx && i0 + tx == 0;
+
+    // ---- phase 1: halo lines; own row -> tile copy and x-line ---------------
+    if (PF && valid && k == 0 && (tx & 1) == 0) {
+        // the low part is first read in phase 4, from HBM when the state
+        // does not fit in L2: start it towards L2 now, one prefetch per
+        // 128-byte line (two elements' rows of one variable)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) asm volatile("prefetch.global.L2 [%0];" ::"l"(A.lo + v * A.npts + e * NN));
+    }
+    Quad x[N], rx[N], eL, fL;
+    if (valid) load_row_quads<N>(A.qs, A.qb, addb, A.npts, off, x);
+    {
+        constexpr int NXH = 2 * TY * N, LINES = NXH + 2 * TX * N;
+        static_assert(LINES <= NT, "at most one halo line per thread");
+        const int t = tid - (NT - LINES);
+        if (active && t >= 0) {
+            const bool xdir = t < NXH;
+            const int r0 = xdir ? t : t - NXH;
+            const int side = r0 >= (xdir ? TY * N : TX * N);
+            const int r = side ? r0 - (xdir ? TY * N : TX * N) : r0;
+            const int pos = r / N, kk = r % N;  // pos: tile row (x) or tile column (y)
+            int gi = xdir ? (side ? i0 + TXe : i0 - 1) : i0 + pos;
+            int gj = xdir ? j0 + pos : (side ? j0 + TYe : j0 - 1);
+            bool have = pos < (xdir ? TYe : TXe);
+            if (gi < 0 || gi >= A.nx) {
+                have = have && !A.bcx;
+                gi = gi < 0 ? gi + A.nx : gi - A.nx;
+            }
+            if (gj < 0 || gj >= A.ny) {
+                have = have && !A.bcy;
+                gj = gj < 0 ? gj + A.ny : gj - A.ny;
+            }
+            if (have) {
+                const long long eh = ((long long)gj * A.nx + gi) * NN;
+                Quad h[N];
+                if (xdir) load_row_quads<N>(A.qs, A.qb, addb, A.npts, eh + kk * N, h);
+                else load_col_quads<N>(A.qs, A.qb, addb, A.npts, eh + kk, h);
+                const Quad es = side ? edge_lo<N>(qt, h) : edge_hi<N>(qt, h);
+                if (xdir) {
+                    if (side) xH[pos * N + kk] = es;
+                    else xR[L::xr(pos, 0, kk)] = es;
+                } else {
+                    if (side) yH[pos * N + kk] = es;
+                    else yT[L::yt(0, pos, kk)] = es;
+                }
+            }
+        }
+    }
+    if (valid) {
+#pragma unroll
+        for (int a = 0; a < N; ++a) sq[L::sq(el, k, a)] = x[a];
+        Quad eR, fR;
+        quad_line<N, 0, DIV>(qt, A.ph, x, rx, eL, eR, fL, fR);
+        xR[L::xr(ty, tx + 1, k)] = eR;
+        xF[L::ef(el, k)] = fR;
+    }
+    // Phase 2 reads only the points of one element from the tile copy.  For
+    // even N the column identity is the row identity and a warp holds whole
+    // elements, so a warp barrier orders its own rows.  Everything else that
+    // phase 1 writes is read after the next CTA barrier.
+    constexpr bool KMAJ = N % 2 == 1;
+    if constexpr (!KMAJ && 32 % N == 0) __syncwarp();
+    else __syncthreads();
+
+    // ---- phase 2: y-line (column kc of element elc) --------------------------
+    const int elc = KMAJ ? tid % (TX * TY) : el, kc = KMAJ ? tid / (TX * TY) : k;
+    const int txc = elc % TX, tyc = elc / TX;
+    const bool validc = active && txc < TXe && tyc < TYe;
+    const bool bwall = A.bcy && j0 + tyc == 0;
+    Quad ry[N], eB, gB;
+    if (validc) {
+        Quad c[N], eT, gT;
+#pragma unroll
+        for (int b = 0; b < N; ++b) c[b] = sq[L::sq(elc, b, kc)];
+        quad_line<N, 1, DIV>(qt, A.ph, c, ry, eB, eT, gB, gT);
+        yT[L::yt(tyc + 1, txc, kc)] = eT;
+        yF[L::ef(elc, kc)] = gT;
+    }
+    __syncthreads();
+
+    // ---- phase 3: common fluxes ----------------------------------------------
+    if (validc) {
+        // lower face: the jump F* - f of this element into its y-derivative,
+        // the neighbour's over its top edge flux
+        const Quad dm = bwall ? eB : yT[L::yt(tyc, txc, kc)];
+        const Quad G = quad_face2<FLUX, 1>(dm, eB, A.ph);
+        const Quad J = half_jump(G, gB);
+        if (tyc > 0) {
+            Quad* pj = yF + L::ef(elc - TX, kc);
+            *pj = half_jump(G, *pj);
+        }
+#pragma unroll
+        for (int b = 0; b < N; ++b) sq[L::sq(elc, b, kc)] = qfma(J, qt.dgl[b], ry[b]);
+    }
+    Quad JL;
+    if (valid) {
+        const Quad dm = lwall ? eL : xR[L::xr(ty, tx, k)];
+        const Quad G = quad_face2<FLUX, 0>(dm, eL, A.ph);
+        JL = half_jump(G, fL);
+        if (tx > 0) {
+            Quad* pj = xF + L::ef(el - 1, k);
+            *pj = half_jump(G, *pj);
+        }
+    }
+    if (tid < (TX + TY) * N) {
+        // right face of the tile's last column (x) / upper face of its last row
+        const bool xe = tid < TY * N;
+        const int r = xe ? tid : tid - TY * N;
+        const int pos = r / N, kk = r % N;
+        if (pos < (xe ? TYe : TXe)) {
+            const bool wall = xe ? (A.bcx && i0 + TXe == A.nx) : (A.bcy && j0 + TYe == A.ny);
+            const Quad Em = xe ? xR[L::xr(pos, TXe, kk)] : yT[L::yt(TYe, pos, kk)];
+            const Quad dp = wall ? Em : (xe ? xH[pos * N + kk] : yH[pos * N + kk]);
+            const Quad G = xe ? quad_face2<FLUX, 0>(Em, dp, A.ph) : quad_face2<FLUX, 1>(Em, dp, A.ph);
+            Quad* pj = xe ? xF + L::ef(pos * TX + TXe - 1, kk) : yF + L::ef((TYe - 1) * TX + pos, kk);
+            *pj = half_jump(G, *pj);
+        }
+    }
+    __syncthreads();
+
+    // ---- phase 4: R on row k, stage update, store ----------------------------
+    float o[4][N];
+    if (valid) {
+        // g_R'(eta_k) = -g_L'(eta_{N-1-k}): one select chain instead of an
+        // indexed parameter load
+        float grk = -qt.dgl[N - 1];
+#pragma unroll
+        for (int b = 1; b < N; ++b) grk = k == b ? -qt.dgl[N - 1 - b] : grk;
+        // the factor of R in the stage's result: dt (increment modes: dt / 4
+        // and 2 dt / 3 of the second and third stage)
+        float w = (float)A.ctrl->dt;
+        if (mode == MODE_INC2) w *= 0.25f;
+        if (mode == MODE_INC3) w *= 2.0f / 3.0f;
+        const float sx = -A.rhx2 * w, sy = -A.rhy2 * w;
+        const Quad JR = xF[L::ef(el, k)];
+#pragma unroll
+        for (int a = 0; a < N; ++a) {
+            Quad y = sq[L::sq(el, k, a)];
+            y = qfma(yF[L::ef(el, a)], grk, y);
+            Quad z = qfma(JL, qt.dgl[a], rx[a]);
+            z = qfma(JR, -qt.dgl[N - 1 - a], z);
+            float yv[4], zv[4];
+            qget(qmul(y, sy), yv);
+            qget(z, zv);
+#pragma unroll
+            for (int v = 0; v < 4; ++v) o[v][a] = fmaf(sx, zv[v], yv[v]);
+        }
+        if (mode == MODE_INC1) {
+        } else if (mode <= MODE_SO3) {
+            const float cA = mode == MODE_SO2 ? 0.75f : 1.0f / 3.0f;
+            const float cB = mode == MODE_SO2 ? 0.25f : 2.0f / 3.0f;
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                float qs[N], qn[N];
+                gload_row<N>(A.qs + v * A.npts + off, qs);
+                if (mode == MODE_SO1) {
+#pragma unroll
+                    for (int a = 0; a < N; ++a) o[v][a] = qs[a] + o[v][a];
+                } else {
+                    gload_row<N>(A.qn + v * A.npts + off, qn);
+#pragma unroll
+                    for (int a = 0; a < N; ++a) o[v][a] = cA * qn[a] + cB * (qs[a] + o[v][a]);
+                }
+            }
+        } else {
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                float b[N];
+                gload_row<N>(A.qb + v * A.npts + off, b);
+                if (mode == MODE_INC2) {
+#pragma unroll
+                    for (int a = 0; a < N; ++a) o[v][a] = fmaf(0.25f, b[a], o[v][a]);
+                } else {
+                    float hi[N], lo[N];
+                    gload_row<N>(A.qs + v * A.npts + off, hi);
+                    gload_row<N>(A.lo + v * A.npts + off, lo);
+#pragma unroll
+                    for (int a = 0; a < N; ++a) {
+                        compensated_add(hi[a], lo[a], fmaf(2.0f / 3.0f, b[a], o[v][a]));
+                        o[v][a] = hi[a];
+                    }
+                    gstore_row<N>(A.lo + v * A.npts + off, lo);
+                }
+            }
+        }
+#pragma unroll
+        for (int v = 0; v < 4; ++v) gstore_row<N>(A.out + v * A.npts + off, o[v]);
+    }
+
+    // ---- fused element averages (Algorithm 9) -----------------------------
+    if (A.do_avg) {
+        if (valid) {
+            float s[4];
+#pragma unroll
+            for (int v = 0; v < 4; ++v) s[v] = line_dot<N>(tb.cavg[k], o[v]);
+            avS[L::ef(el, k)] = qput(s);
+        }
+        __syncthreads();
+        const int ax = tid % TX, ay = tid / TX;
+        if (tid < TX * TY && ax < TXe && ay < TYe) {
+            Quad s = avS[L::ef(tid, 0)];
+#pragma unroll
+            for (int b = 1; b < N; ++b) s = qadd(s, avS[L::ef(tid, b)]);
+            float sv[4];
+            qget(s, sv);
+            const long long ne = A.npts / NN, ea = (long long)(j0 + ay) * A.nx + (i0 + ax);
+#pragma unroll
+            for (int v = 0; v < 4; ++v) A.avg[v * ne + ea] = sv[v];
+        }
+    }
+
+    // ---- fused max signal speed for the next CFL step ---------------------
+    // (only CFL runs need the speed; a run of fixed steps only closes the
+    // step; the branch is uniform over the grid)
+    if (A.do_wave) {
+        const bool cfl = !(A.ctrl->dt_fixed > 0.0);
+        float m = 0.f;
+        if (cfl && valid) {
+#pragma unroll
+            for (int a = 0; a < N; ++a) {
+                const float q[4] = {o[0][a], o[1][a], o[2][a], o[3][a]};
+                const float s = point_speed<EQ_EULER, true>(q, A.ph);
+                m = s > m ? s : m;
+            }
+        }
+        block_time_update<float>(m, A.ctrl, /*advance=*/true, nslots, cfl);
+    }
+}
+
+// Resident CTAs per SM of a single problem's kernels.  p = 4: 4 CTAs of 32
+// elements (94 registers, no spills) instead of the 6 (64 registers, 44 bytes
+// of spills) that batches keep: 821 x 819 p = 4 303 -> 281 us per stage, the
+// 64-instance batch 31.5 -> 32.5 ms per 24 steps.
+template <int P, bool WIDE, int ELEMS>
+constexpr int quad_min_blocks()
+{
+    return P == 4 && !WIDE ? 128 / ELEMS : stage_min_blocks<float, P + 1, WIDE, ELEMS>();
+}
+
+template <int P, int DIV, int FLUX, int TX, int TY, int MINB, int MODE>
+__global__ void __launch_bounds__(TX * TY * (P + 1), MINB) cpr_stage_quad_kernel(const StageArgs<float> A)
+{
+    static_assert((TX * TY * (P + 1)) % 32 == 0, "whole warps: the warp-level reductions use every lane");
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    stage_tile_quad<P, DIV, FLUX, TX, TY, false, MODE>(A, A.tab, A.qx, blockIdx.x, threadIdx.x, smem_raw, gridDim.x);
+}
+
+}  // namespace cpr

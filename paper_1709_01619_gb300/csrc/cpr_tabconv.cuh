@@ -50,4 +50,28 @@ inline TabPr<T> host_tabpr(const HostTab& h)
     return t;
 }
 
+// The tables of the quad form (QuadTab), formed in FP64.
+inline QuadTab host_quadtab(const HostTab& h)
+{
+    QuadTab t{};
+    const int n = h.n;
+    for (int a = 0; a < n; ++a) {
+        t.lm[a] = float(h.lm[a]);
+        t.dgl[a] = float(h.dgl[a]);
+    }
+    for (int a = 0; a < (n + 1) / 2; ++a) {
+        auto C = [&](int m) {
+            double s = 0.0;
+            for (int l = n - 1; l > m; --l) s += h.D[a][l];
+            return s;
+        };
+        for (int m = 0; m < (n - 1) / 2; ++m) {
+            t.ce[a][m] = float(0.5 * (C(m) + C(n - 2 - m)));
+            t.co[a][m] = float(0.5 * (C(m) - C(n - 2 - m)));
+        }
+        if (n % 2 == 0) t.cm[a] = float(C(n / 2 - 1));
+    }
+    return t;
+}
+
 }  // namespace cpr
