@@ -958,8 +958,11 @@ extern "C" cpr_status cpr_batch_tune(cpr_batch* b, void* const* q, int* choices,
         g.grid = best_grid;
     }
     // The grouped launches just chosen against per-instance chains (stages 1
-    // and 2 of every instance, each form captured in a graph and timed over
-    // three replays).
+    // and 2 of every instance, kTuneSteps times in a graph, timed over three
+    // replays).  Several steps, because the chains join only at the end of a
+    // graph: with one step the joins hid their gain and either form could win
+    // (64 instances, 24 steps: 31.8 ms per-instance, 33.1 ms grouped).
+    const int kTuneSteps = 4;
     {
         auto timed = [&](bool inst, float* ms) -> cudaError_t {
             cudaGraph_t gr = nullptr;
@@ -970,10 +973,10 @@ extern "C" cpr_status cpr_batch_tune(cpr_batch* b, void* const* q, int* choices,
             if (e != cudaSuccess) return e;
             cudaError_t ee = cudaSuccess;
             if (inst) {
-                ee = enqueue_inst_chains(b, 1, b->cap, true);
+                ee = enqueue_inst_chains(b, kTuneSteps, b->cap, true);
             } else {
-                for (int m = 0; m < 2 && ee == cudaSuccess; ++m) {
-                    const int mode = b->use_inc ? modes_inc[m] : modes_so[m];
+                for (int m = 0; m < 2 * kTuneSteps && ee == cudaSuccess; ++m) {
+                    const int mode = b->use_inc ? modes_inc[m % 2] : modes_so[m % 2];
                     for (Group& g : b->groups) {
                         ee = b->dtype == CPR_F32 ? batch_launch<float>(b, g, g.fam, g.grid, mode, 0, b->cap)
                                                  : batch_launch<double>(b, g, g.fam, g.grid, mode, 0, b->cap);
