@@ -14,24 +14,36 @@
 // on the same five-element stencil.  Ghost elements: periodic directions
 // wrap, transmissive ones repeat the boundary element.
 //
-// CTA: a tile of 32 x 8 elements, one thread per element.  Phase 1 stages
-// the tile with a ring of two elements in shared memory; phase 2 evaluates
-// every face of the tile once (the faces on the tile boundary are also
-// evaluated by the neighbouring CTA, from the same values and in the same
-// order, so the flux leaving one element is the flux entering the next);
-// phase 3 forms the residual, applies the RK stage (the modes of the CPR
-// stage kernel) and stores, with the fused maximum signal speed on the last
-// stage.
+// One warp owns a strip of 28 columns of elements (lanes 2..29; the outer two
+// lanes of either side are the ring of the reconstruction) and walks up its
+// rows.  Along y everything a row shares with the one below it (the element
+// values, the difference, the upper face state and the flux of the face
+// between them) stays in registers; along x the neighbour values, the lower
+// state and the flux of the right face come from the next lane by shuffle.
+// So a face of the strip is evaluated once, nothing goes through shared
+// memory and no barrier separates the phases; the next row's values are
+// loaded one row ahead.  Faces on the strip's boundary are also evaluated by
+// the neighbouring warp, from the same values and in the same order, so the
+// flux leaving one element is the flux entering the next.
+//
+// The kernel is bound by the instructions of a row and their latency.  A tile
+// of 32 x 8 elements per CTA, staged in shared memory with its ring, took a
+// second, nearly empty pass over the faces (33 x 8 of them for 256 threads),
+// three barriers and twice the instructions: 1536^2, second order, 12 FP32
+// steps 2.44 -> 1.33 ms (67.7 -> 37.0 us per stage; 1.48 -> 2.72 TB/s of the
+// eight state arrays that a step has to move).
 #pragma once
 
 #include "cpr_common.cuh"
 #include "cpr_launch.h"
 #include "cpr_reduce.cuh"
 #include "cpr_stage.cuh"
+#include "cpr_stage_quad.cuh"
 
 namespace cpr {
 
-constexpr int kFvTX = 32, kFvTY = 8;
+constexpr int kFvCols = 28;   // columns of elements per warp
+constexpr int kFvWarps = 4;   // warps per CTA: neighbouring strips, whose rings overlap in L1
 
 // Wrapped (periodic) or clamped (transmissive) element index, for indices
 // at most two outside [0, n) (no integer division: n may be 1).
@@ -43,143 +55,275 @@ __device__ __forceinline__ int fv_ghost(int i, int n, int transmissive)
     return i;
 }
 
-// Face states of element b (neighbours a below, c above along the line):
-// its value on the upper face (up) and on the lower face (down).
-template <int ORDER, class T>
-__device__ __forceinline__ T fv_up(T a, T b, T c)
+// Minmod of the slopes.  FP32: the minimum if both are positive plus the
+// maximum if both are negative.  FP64 (comparisons run on the FP64 pipe): one
+// comparison of the magnitudes and the signs from the high words.
+__device__ __forceinline__ float fv_minmod(float a, float b)
 {
-    if constexpr (ORDER == 2) {
-        return b + T(0.5) * minmod2(c - b, b - a);
+    return fmaxf(fminf(a, b), 0.f) + fminf(fmaxf(a, b), 0.f);
+}
+__device__ __forceinline__ double fv_minmod(double a, double b)
+{
+    const double m = ::fabs(a) < ::fabs(b) ? a : b;
+    return (__double2hiint(a) ^ __double2hiint(b)) < 0 ? 0.0 : m;
+}
+
+// The variables of one element.
+template <class T, int V>
+struct FvEl {
+    T v[V];
+};
+template <class T, int V>
+__device__ __forceinline__ FvEl<T, V> fv_up_lane(const FvEl<T, V>& x)  // the value of the lane below
+{
+    FvEl<T, V> r;
+#pragma unroll
+    for (int k = 0; k < V; ++k) r.v[k] = __shfl_up_sync(0xffffffffu, x.v[k], 1);
+    return r;
+}
+template <class T, int V>
+__device__ __forceinline__ FvEl<T, V> fv_down_lane(const FvEl<T, V>& x)
+{
+    FvEl<T, V> r;
+#pragma unroll
+    for (int k = 0; k < V; ++k) r.v[k] = __shfl_down_sync(0xffffffffu, x.v[k], 1);
+    return r;
+}
+
+// c x + y; FP32 Euler in packed pairs.
+template <class T, int V>
+__device__ __forceinline__ FvEl<T, V> fv_axpy(T c, const FvEl<T, V>& x, const FvEl<T, V>& y)
+{
+    FvEl<T, V> r;
+    if constexpr (V == 4) {
+        qget(qfma(qput(x.v), c, qput(y.v)), r.v);
     } else {
-        const T dm = b - a, dp = c - b;
-        return b + (minmod2(dm, T(4) * dp) * T(1.0 / 6.0) + minmod2(dp, T(4) * dm) * T(1.0 / 3.0));
+#pragma unroll
+        for (int k = 0; k < V; ++k) r.v[k] = fma(c, x.v[k], y.v[k]);
+    }
+    return r;
+}
+// a - b (exact as -1 b + a)
+template <class T, int V>
+__device__ __forceinline__ FvEl<T, V> fv_diff(const FvEl<T, V>& a, const FvEl<T, V>& b) { return fv_axpy(T(-1), b, a); }
+template <class T, int V>
+__device__ __forceinline__ FvEl<T, V> fv_scale(T c, const FvEl<T, V>& x)
+{
+    FvEl<T, V> r;
+    if constexpr (V == 4) {
+        qget(qmul(qput(x.v), c), r.v);
+    } else {
+#pragma unroll
+        for (int k = 0; k < V; ++k) r.v[k] = c * x.v[k];
+    }
+    return r;
+}
+
+// Face states of element b with the one-sided differences dm, dp along the
+// line: its value on the upper face (up) and on the lower face (dn).
+template <int ORDER, class T, int V>
+__device__ __forceinline__ void fv_states(const FvEl<T, V>& b, const FvEl<T, V>& dm, const FvEl<T, V>& dp,
+                                          FvEl<T, V>& up, FvEl<T, V>& dn)
+{
+#pragma unroll
+    for (int k = 0; k < V; ++k) {
+        if constexpr (ORDER == 2) {
+            up.v[k] = fv_minmod(dp.v[k], dm.v[k]);
+        } else {
+            const T m1 = fv_minmod(dm.v[k], T(4) * dp.v[k]), m2 = fv_minmod(dp.v[k], T(4) * dm.v[k]);
+            up.v[k] = b.v[k] + fma(m1, T(1.0 / 6.0), m2 * T(1.0 / 3.0));
+            dn.v[k] = b.v[k] - fma(m2, T(1.0 / 6.0), m1 * T(1.0 / 3.0));
+        }
+    }
+    if constexpr (ORDER == 2) {
+        const FvEl<T, V> s = up;
+        up = fv_axpy(T(0.5), s, b);
+        dn = fv_axpy(T(-0.5), s, b);
     }
 }
-template <int ORDER, class T>
-__device__ __forceinline__ T fv_down(T a, T b, T c)
+
+// Twice the common flux between the lower state m and the upper state p.
+template <int EQ, int FLUX, int DIR, class T, int V>
+__device__ __forceinline__ FvEl<T, V> fv_face2(const FvEl<T, V>& m, const FvEl<T, V>& p, const Phys<T>& ph)
 {
-    if constexpr (ORDER == 2) {
-        return b - T(0.5) * minmod2(c - b, b - a);
+    FvEl<T, V> F;
+    if constexpr (EQ == EQ_EULER) {
+        qget(quad_face2<FLUX, DIR>(qput(m.v), qput(p.v), ph), F.v);
     } else {
-        const T dm = b - a, dp = c - b;
-        return b - (minmod2(dp, T(4) * dm) * T(1.0 / 6.0) + minmod2(dm, T(4) * dp) * T(1.0 / 3.0));
+        common_flux<EQ, FLUX, DIR>(m.v, p.v, ph, F.v);
+        F.v[0] *= T(2);
     }
+    return F;
+}
+
+// Resident CTAs the register budget is sized for: FP32 six, 24 warps per SM
+// (80 registers, no spills).  1536^2, us per stage: five CTAs 44, six 37, seven
+// (72 registers) 41.
+constexpr int kFvResident = 6;
+template <class T>
+constexpr int fv_min_blocks()
+{
+    return sizeof(T) == 4 ? kFvResident : 1;
+}
+
+// MODE: the stage mode, or -1 for the one in the arguments.
+template <class T, int EQ, int FLUX, int ORDER, int MODE>
+__global__ void __launch_bounds__(kFvWarps * 32, fv_min_blocks<T>())
+cpr_fv_stage_kernel(const StageArgs<T> A, const int rows)
+{
+    constexpr int V = NVars<EQ>::value;
+    using El = FvEl<T, V>;
+    const int mode = MODE >= 0 ? MODE : A.mode;
+    if (mode > 0 && A.ctrl->done) return;  // t_end reached: uniform exit
+    const int lane = threadIdx.x & 31;
+    // rows by CTA, so that every row pointer is uniform over the CTA
+    const int by = blockIdx.x / A.tiles_x, j0 = by * rows, jend = min(j0 + rows, A.ny);
+    const int i0 = ((blockIdx.x - by * A.tiles_x) * kFvWarps + (threadIdx.x >> 5)) * kFvCols;
+    const int col = i0 + lane - 2;
+    const bool valid = lane >= 2 && lane < 2 + kFvCols && col < A.nx;
+    const bool addb = mode == MODE_INC2 || mode == MODE_INC3;
+    // lanes past the ring of a ragged strip repeat its last column
+    const unsigned int gi = (unsigned int)fv_ghost(min(col, A.nx + 1), A.nx, A.bcx);
+    T m = T(0);
+
+    if (i0 < A.nx) {
+        auto row_of = [&](const T* p, int j) {
+            El x;
+            p += (long long)j * A.nx;
+#pragma unroll
+            for (int v = 0; v < V; ++v) x.v[v] = (p + v * A.npts)[gi];
+            return x;
+        };
+        El nq, nb;  // the row being loaded: state and increment
+        auto fetch = [&](int j) {
+            j = fv_ghost(j, A.ny, A.bcy);
+            nq = row_of(A.qs, j);
+            if (addb) nb = row_of(A.qb, j);
+        };
+        auto row = [&]() { return addb ? fv_axpy(T(1), nq, nb) : nq; };
+        fetch(j0 - 2);
+        const El a = row();
+        fetch(j0 - 1);
+        El c = row();
+        fetch(j0);
+        El d = row();
+        fetch(j0 + 1);
+        El upl, up, dn;           // upl: upper state of row j
+        El dyn = fv_diff(d, c);   // difference across the upper face of row j
+        El Glo{};                 // flux of the lower face of row j
+        fv_states<ORDER>(c, fv_diff(c, a), dyn, upl, dn);
+
+        // the factor of R in the stage's result
+        T w = mode > 0 ? T(A.ctrl->dt) : T(1);
+        if (mode == MODE_SO2 || mode == MODE_INC2) w *= T(0.25);
+        if (mode == MODE_SO3 || mode == MODE_INC3) w *= T(2.0 / 3.0);
+        // one half of 1 / dx, 1 / dy: the fluxes are doubled
+        const T sx = T(-0.25) * A.rhx2 * w, sy = T(-0.25) * A.rhy2 * w;
+        // row j0 - 1 is there for its upper face only (the same instructions
+        // for every face, so that both warps of a face see the same bits)
+        for (int j = j0 - 1; j < jend; ++j) {
+            const El n = row();  // row j + 2
+            if (j + 1 < jend) fetch(j + 3);
+            const int jo = max(j, j0);
+            El s0, s1, s2;  // what the stage update adds: started here, used last
+            if (mode >= MODE_SO1 && mode != MODE_INC1) s0 = row_of(mode == MODE_INC2 ? A.qb : A.qs, jo);
+            if (mode == MODE_SO2 || mode == MODE_SO3) s1 = row_of(A.qn, jo);
+            if (mode == MODE_INC3) {
+                s1 = row_of(A.qb, jo);
+                s2 = row_of(A.lo, jo);
+            }
+            // upper face of the row
+            const El dnn = fv_diff(n, d);
+            fv_states<ORDER>(d, dyn, dnn, up, dn);
+            const El Ghi = fv_face2<EQ, FLUX, 1>(upl, dn, A.ph);
+            upl = up;
+            // left face, and the right one from the next lane
+            const El dx = fv_diff(c, fv_up_lane(c));
+            fv_states<ORDER>(c, dx, fv_down_lane(dx), up, dn);
+            const El Fl = fv_face2<EQ, FLUX, 0>(fv_up_lane(up), dn, A.ph);
+            El o = fv_scale(sx, fv_diff(fv_down_lane(Fl), Fl));
+            o = fv_axpy(sy, fv_diff(Ghi, Glo), o);
+            if (mode == MODE_SO1) {
+                o = fv_axpy(T(1), s0, o);
+            } else if (mode == MODE_SO2 || mode == MODE_SO3) {
+                o = fv_axpy(mode == MODE_SO2 ? T(0.75) : T(1.0 / 3.0), s1,
+                            fv_axpy(mode == MODE_SO2 ? T(0.25) : T(2.0 / 3.0), s0, o));
+            } else if (mode == MODE_INC2) {
+                o = fv_axpy(T(0.25), s0, o);
+            } else if (mode == MODE_INC3) {
+                o = fv_axpy(T(2.0 / 3.0), s1, o);
+#pragma unroll
+                for (int v = 0; v < V; ++v) {
+                    compensated_add(s0.v[v], s2.v[v], o.v[v]);
+                    o.v[v] = s0.v[v];
+                }
+            }
+            if (valid && j >= j0) {
+                const long long r0 = (long long)j * A.nx;
+#pragma unroll
+                for (int v = 0; v < V; ++v) {
+                    (A.out + v * A.npts + r0)[gi] = o.v[v];
+                    if (mode == MODE_INC3) (A.lo + v * A.npts + r0)[gi] = s2.v[v];
+                }
+                if (A.do_wave) {
+                    const T sp = point_speed<EQ, true>(o.v, A.ph);
+                    m = sp > m ? sp : m;
+                }
+            }
+            c = d;
+            d = n;
+            dyn = dnn;
+            Glo = Ghi;
+        }
+    }
+    if (A.do_wave) block_time_update<T>(m, A.ctrl, /*advance=*/true, gridDim.x);
+}
+
+// Rows per strip: a strip costs about two rows beyond its own, and the pass
+// takes the time of the SM with most CTAs; a row takes 0.6 us plus 0.14 us for
+// every CTA that shares its SM, so few tall strips leave the SM waiting.  Of
+// the heights that give every SM almost its resident CTAs or more, the one with
+// the fewest rows on the busiest SM (1536^2: 24 rows, six CTAs each; 37 us per
+// stage, 36 rows and four CTAs 50); smaller grids take two rows.
+inline int fv_rows(int ctas_x, int ny, int sms)
+{
+    constexpr int kMaxRows = 48;
+    int best = 2;
+    long long cost = -1;
+    for (int r = 2; r <= kMaxRows; ++r) {
+        const long long ctas = (long long)ctas_x * ((ny + r - 1) / r);
+        if (r > 2 && ctas < (long long)(kFvResident - 1) * sms) break;
+        const long long c = (ctas + sms - 1) / sms * (r + 2);
+        if (cost < 0 || c <= cost) {
+            best = r;
+            cost = c;
+        }
+    }
+    return best;
 }
 
 template <class T, int EQ, int FLUX, int ORDER>
-__global__ void __launch_bounds__(kFvTX * kFvTY) cpr_fv_stage_kernel(const StageArgs<T> A)
+static cudaError_t fv_order(const LaunchCfg& c, const StageArgs<T>& A, cudaStream_t s)
 {
-    constexpr int TX = kFvTX, TY = kFvTY, NT = TX * TY, HX = TX + 4, HY = TY + 4;
-    constexpr int V = NVars<EQ>::value;
-    __shared__ T s[V][HY][HX];           // tile and two-element ring; s[v][ly][lx] = element (lx-2, ly-2)
-    __shared__ T fx[V][TY][TX + 1];      // x-face fluxes; face fi between elements fi-1 and fi
-    __shared__ T gy[V][TY + 1][TX];      // y-face fluxes; face fj between elements fj-1 and fj
-
-    if (A.mode > 0 && A.ctrl->done) return;  // t_end reached: uniform exit
-    const int tid = threadIdx.x;
-    const int i0 = (blockIdx.x % A.tiles_x) * TX, j0 = (blockIdx.x / A.tiles_x) * TY;
-    const int TXe = min(TX, A.nx - i0), TYe = min(TY, A.ny - j0);
-    const bool addb = A.mode == MODE_INC2 || A.mode == MODE_INC3;
-
-    // ---- phase 1: stage input of the tile and its ring --------------------
-    for (int t = tid; t < HX * HY; t += NT) {
-        const int lx = t % HX, ly = t / HX;
-        const int gi = fv_ghost(i0 + lx - 2, A.nx, A.bcx), gj = fv_ghost(j0 + ly - 2, A.ny, A.bcy);
-        const long long e = (long long)gj * A.nx + gi;
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-            T x = A.qs[v * A.npts + e];
-            if (addb) x += A.qb[v * A.npts + e];
-            s[v][ly][lx] = x;
-        }
+    const int rows = fv_rows(A.tiles_x, c.ny, c.sms > 0 ? c.sms : 1);
+    const int ctas = A.tiles_x * ((c.ny + rows - 1) / rows);
+    auto launch = [&](auto k) {
+        k<<<ctas, kFvWarps * 32, 0, s>>>(A, rows);
+        return cudaGetLastError();
+    };
+    // FP32 steps take a kernel compiled for their stage mode
+    if constexpr (sizeof(T) == 4) {
+        if (A.mode == MODE_INC1) return launch(cpr_fv_stage_kernel<T, EQ, FLUX, ORDER, MODE_INC1>);
+        if (A.mode == MODE_INC2) return launch(cpr_fv_stage_kernel<T, EQ, FLUX, ORDER, MODE_INC2>);
+        if (A.mode == MODE_INC3) return launch(cpr_fv_stage_kernel<T, EQ, FLUX, ORDER, MODE_INC3>);
     }
-    __syncthreads();
-
-    // ---- phase 2: reconstruction and common flux on every face -------------
-    for (int f = tid; f < (TX + 1) * TY; f += NT) {
-        const int fi = f % (TX + 1), fj = f / (TX + 1);
-        if (fi > TXe || fj >= TYe) continue;
-        T qm[V], qp[V], F[V];
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-            const T* r = &s[v][fj + 2][fi];  // elements fi-2 .. fi+1
-            qm[v] = fv_up<ORDER>(r[0], r[1], r[2]);
-            qp[v] = fv_down<ORDER>(r[1], r[2], r[3]);
-        }
-        common_flux<EQ, FLUX, 0>(qm, qp, A.ph, F);
-#pragma unroll
-        for (int v = 0; v < V; ++v) fx[v][fj][fi] = F[v];
-    }
-    for (int f = tid; f < TX * (TY + 1); f += NT) {
-        const int fi = f % TX, fj = f / TX;
-        if (fi >= TXe || fj > TYe) continue;
-        T qm[V], qp[V], F[V];
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-            const T a = s[v][fj][fi + 2], b = s[v][fj + 1][fi + 2], c = s[v][fj + 2][fi + 2],
-                    d = s[v][fj + 3][fi + 2];  // elements fj-2 .. fj+1
-            qm[v] = fv_up<ORDER>(a, b, c);
-            qp[v] = fv_down<ORDER>(b, c, d);
-        }
-        common_flux<EQ, FLUX, 1>(qm, qp, A.ph, F);
-#pragma unroll
-        for (int v = 0; v < V; ++v) gy[v][fj][fi] = F[v];
-    }
-    __syncthreads();
-
-    // ---- phase 3: residual, stage update, store -----------------------------
-    const int tx = tid % TX, ty = tid / TX;
-    const bool valid = tx < TXe && ty < TYe;
-    T o[V];
-    if (valid) {
-        const T ihx = T(0.5) * A.rhx2, ihy = T(0.5) * A.rhy2;  // 1/dx, 1/dy
-        const long long e = (long long)(j0 + ty) * A.nx + (i0 + tx);
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-            const T r = -(fx[v][ty][tx + 1] - fx[v][ty][tx]) * ihx - (gy[v][ty + 1][tx] - gy[v][ty][tx]) * ihy;
-            const long long k = v * A.npts + e;
-            T y = r;
-            if (A.mode == MODE_RESIDUAL) {
-            } else if (A.mode <= MODE_SO3) {
-                const T dt = T(A.ctrl->dt);
-                const T qs = A.qs[k];
-                if (A.mode == MODE_SO1) {
-                    y = qs + dt * r;
-                } else {
-                    const T cA = A.mode == MODE_SO2 ? T(0.75) : T(1.0 / 3.0);
-                    const T cB = A.mode == MODE_SO2 ? T(0.25) : T(2.0 / 3.0);
-                    y = cA * A.qn[k] + cB * (qs + dt * r);
-                }
-            } else {
-                const T dt = T(A.ctrl->dt);
-                if (A.mode == MODE_INC1) {
-                    y = dt * r;
-                } else if (A.mode == MODE_INC2) {
-                    y = T(0.25) * (A.qb[k] + dt * r);
-                } else {
-                    T hi = A.qs[k], lo = A.lo[k];
-                    compensated_add(hi, lo, T(2.0 / 3.0) * (A.qb[k] + dt * r));
-                    A.lo[k] = lo;
-                    y = hi;
-                }
-            }
-            A.out[k] = y;
-            o[v] = y;
-        }
-    }
-    if (A.do_wave) {
-        T m = valid ? point_speed<EQ>(o, A.ph) : T(0);
-        block_time_update<T>(m, A.ctrl, /*advance=*/true, gridDim.x);
-    }
+    return launch(cpr_fv_stage_kernel<T, EQ, FLUX, ORDER, -1>);
 }
 
 template <class T, int EQ, int FLUX>
 static cudaError_t fv_one(const LaunchCfg& c, const StageArgs<T>& A, cudaStream_t s)
 {
-    const int ctas = ((c.nx + kFvTX - 1) / kFvTX) * ((c.ny + kFvTY - 1) / kFvTY);
-    if (c.fv_order == 3) cpr_fv_stage_kernel<T, EQ, FLUX, 3><<<ctas, kFvTX * kFvTY, 0, s>>>(A);
-    else cpr_fv_stage_kernel<T, EQ, FLUX, 2><<<ctas, kFvTX * kFvTY, 0, s>>>(A);
-    return cudaGetLastError();
+    return c.fv_order == 3 ? fv_order<T, EQ, FLUX, 3>(c, A, s) : fv_order<T, EQ, FLUX, 2>(c, A, s);
 }
 
 }  // namespace cpr

@@ -380,7 +380,7 @@ constexpr bool stage_quad = sizeof(T) == 4 && EQ == EQ_EULER && !DELTA;
 template <class T, int P, int EQ, int TX, int TY, bool DELTA>
 constexpr size_t stage_smem()
 {
-    if constexpr (stage_quad<T, EQ, DELTA>) return sizeof(Quad) * QuadLayout<P + 1, TX, TY>::TOTAL;
+    if constexpr (stage_quad<T, EQ, DELTA>) return sizeof(Quad<float>) * QuadLayout<P + 1, TX, TY>::TOTAL;
     else return sizeof(T) * StageLayout<P + 1, NVars<EQ>::value, TX, TY, DELTA>::TOTAL;
 }
 

@@ -20,43 +20,51 @@
 
 namespace cpr {
 
+template <class T>
 struct alignas(16) Quad {
-    Pr<float> a, b;  // (rho, rho u), (rho v, e)
+    Pr<T> a, b;  // (rho, rho u), (rho v, e)
 };
 
-__device__ __forceinline__ Quad qmk(float x, float y, float z, float w) { return {pmk(x, y), pmk(z, w)}; }
-__device__ __forceinline__ Quad qmul(const Quad& x, float c) { return {pmul(pbc(c), x.a), pmul(pbc(c), x.b)}; }
-__device__ __forceinline__ Quad qfma(const Quad& x, float c, const Quad& y)
+template <class T>
+__device__ __forceinline__ Quad<T> qmk(T x, T y, T z, T w) { return {pmk(x, y), pmk(z, w)}; }
+template <class T>
+__device__ __forceinline__ Quad<T> qmul(const Quad<T>& x, T c) { return {pmul(pbc(c), x.a), pmul(pbc(c), x.b)}; }
+template <class T>
+__device__ __forceinline__ Quad<T> qfma(const Quad<T>& x, T c, const Quad<T>& y)
 {
     return {pfma(pbc(c), x.a, y.a), pfma(pbc(c), x.b, y.b)};
 }
-__device__ __forceinline__ Quad qadd(const Quad& x, const Quad& y) { return {padd(x.a, y.a), padd(x.b, y.b)}; }
-__device__ __forceinline__ Quad qsub(const Quad& x, const Quad& y) { return {psub(x.a, y.a), psub(x.b, y.b)}; }
-__device__ __forceinline__ void qget(const Quad& x, float* v)
+template <class T>
+__device__ __forceinline__ Quad<T> qadd(const Quad<T>& x, const Quad<T>& y) { return {padd(x.a, y.a), padd(x.b, y.b)}; }
+template <class T>
+__device__ __forceinline__ Quad<T> qsub(const Quad<T>& x, const Quad<T>& y) { return {psub(x.a, y.a), psub(x.b, y.b)}; }
+template <class T>
+__device__ __forceinline__ void qget(const Quad<T>& x, T* v)
 {
     v[0] = x.a.v.x;
     v[1] = x.a.v.y;
     v[2] = x.b.v.x;
     v[3] = x.b.v.y;
 }
-__device__ __forceinline__ Quad qput(const float* v) { return qmk(v[0], v[1], v[2], v[3]); }
+template <class T>
+__device__ __forceinline__ Quad<T> qput(const T* v) { return qmk(v[0], v[1], v[2], v[3]); }
 
 // Edge states of a line of N quads at -1 (lo) and +1 (hi).  The solution
 // points are symmetric, so l_l(+1) = l_{N-1-l}(-1): one table serves both.
 // Every edge state of the kernel, the element's own and the one a neighbour
 // CTA forms from its halo line, is one of these two sums in this order.
 template <int N>
-__device__ __forceinline__ Quad edge_lo(const QuadTab& t, const Quad (&x)[N])
+__device__ __forceinline__ Quad<float> edge_lo(const QuadTab& t, const Quad<float> (&x)[N])
 {
-    Quad s = qmul(x[0], t.lm[0]);
+    Quad<float> s = qmul(x[0], t.lm[0]);
 #pragma unroll
     for (int l = 1; l < N; ++l) s = qfma(x[l], t.lm[l], s);
     return s;
 }
 template <int N>
-__device__ __forceinline__ Quad edge_hi(const QuadTab& t, const Quad (&x)[N])
+__device__ __forceinline__ Quad<float> edge_hi(const QuadTab& t, const Quad<float> (&x)[N])
 {
-    Quad s = qmul(x[N - 1], t.lm[0]);
+    Quad<float> s = qmul(x[N - 1], t.lm[0]);
 #pragma unroll
     for (int l = 1; l < N; ++l) s = qfma(x[N - 1 - l], t.lm[l], s);
     return s;
@@ -70,20 +78,20 @@ __device__ __forceinline__ Quad edge_hi(const QuadTab& t, const Quad (&x)[N])
 // two points at once: 8 / 13 / 22 operations per pair of variables for
 // N = 3 / 4 / 5 against 9 / 16 / 25 of the row sums.
 template <int N>
-__device__ __forceinline__ void line_derivative(const QuadTab& t, const Quad (&f)[N], Quad (&r)[N])
+__device__ __forceinline__ void line_derivative(const QuadTab& t, const Quad<float> (&f)[N], Quad<float> (&r)[N])
 {
     constexpr int M = N - 1, H = M / 2;
-    Quad s[H > 0 ? H : 1], d[H > 0 ? H : 1], mid;
+    Quad<float> s[H > 0 ? H : 1], d[H > 0 ? H : 1], mid;
 #pragma unroll
     for (int m = 0; m < H; ++m) {
-        const Quad lo = qsub(f[m + 1], f[m]), hi = qsub(f[N - 1 - m], f[N - 2 - m]);
+        const Quad<float> lo = qsub(f[m + 1], f[m]), hi = qsub(f[N - 1 - m], f[N - 2 - m]);
         s[m] = qadd(lo, hi);
         d[m] = qsub(lo, hi);
     }
     if constexpr (M % 2 == 1) mid = qsub(f[H + 1], f[H]);
 #pragma unroll
     for (int a = 0; a < (N + 1) / 2; ++a) {
-        Quad p;
+        Quad<float> p;
         if constexpr (M % 2 == 1) {
             p = qmul(mid, t.cm[a]);
 #pragma unroll
@@ -96,7 +104,7 @@ __device__ __forceinline__ void line_derivative(const QuadTab& t, const Quad (&f
         if (2 * a == N - 1) {
             r[a] = p;
         } else {
-            Quad lo = p, hi = p;
+            Quad<float> lo = p, hi = p;
 #pragma unroll
             for (int m = 0; m < H; ++m) {
                 lo = qfma(d[m], t.co[a][m], lo);
@@ -143,7 +151,7 @@ struct QuadLayout {
 // the increment array.
 template <int N>
 __device__ __forceinline__ void load_row_quads(const float* __restrict__ q, const float* __restrict__ qb, bool addb,
-                                               long long npts, long long off, Quad (&x)[N])
+                                               long long npts, long long off, Quad<float> (&x)[N])
 {
     float r[4][N];
 #pragma unroll
@@ -164,7 +172,7 @@ __device__ __forceinline__ void load_row_quads(const float* __restrict__ q, cons
 // Column of N values (stride N) of every variable as quads.
 template <int N>
 __device__ __forceinline__ void load_col_quads(const float* __restrict__ q, const float* __restrict__ qb, bool addb,
-                                               long long npts, long long off, Quad (&x)[N])
+                                               long long npts, long long off, Quad<float> (&x)[N])
 {
     float r[4][N];
 #pragma unroll
@@ -188,48 +196,49 @@ __device__ __forceinline__ void load_col_quads(const float* __restrict__ q, cons
 
 // Flux of Eq. 4 through DIR at one point; SPEED: also the signal speed
 // |Vn| + c.
-template <int DIR, bool SPEED = false>
-__device__ __forceinline__ Quad quad_flux(const Quad& q, const Phys<float>& ph, float* s = nullptr)
+template <int DIR, bool SPEED = false, class T>
+__device__ __forceinline__ Quad<T> quad_flux(const Quad<T>& q, const Phys<T>& ph, T* s = nullptr)
 {
-    float v[4], u, w, r;
+    T v[4], u, w, r;
     qget(q, v);
-    const float p = pressure<true>(v, ph.gamma, u, w, r);
-    const float vn = DIR == 0 ? u : w;
-    if constexpr (SPEED) *s = fabsf(vn) + fsqrt_ftz(ph.gamma * p * r);
-    const float h = (v[3] + p) * vn;
-    if constexpr (DIR == 0) return qmk(v[1], fmaf(v[1], u, p), v[2] * u, h);
-    else return qmk(v[2], v[1] * w, fmaf(v[2], w, p), h);
+    const T p = pressure<true>(v, ph.gamma, u, w, r);
+    const T vn = DIR == 0 ? u : w;
+    if constexpr (SPEED) *s = ::fabs(vn) + sqrt_of<true>(ph.gamma * p * r);
+    const T h = (v[3] + p) * vn;
+    if constexpr (DIR == 0) return qmk(v[1], fma(v[1], u, p), v[2] * u, h);
+    else return qmk(v[2], v[1] * w, fma(v[2], w, p), h);
 }
 
 // Twice the common flux through a face between the lower state m and the
 // upper state p (the factor 1/2 joins the jump's subtraction, half_jump).
-template <int FLUX, int DIR>
-__device__ __forceinline__ Quad quad_face2(const Quad& m, const Quad& p, const Phys<float>& ph)
+template <int FLUX, int DIR, class T>
+__device__ __forceinline__ Quad<T> quad_face2(const Quad<T>& m, const Quad<T>& p, const Phys<T>& ph)
 {
     if constexpr (FLUX == FLUX_RUSANOV) {
-        float sm, sp;
-        const Quad fm = quad_flux<DIR, true>(m, ph, &sm), fp = quad_flux<DIR, true>(p, ph, &sp);
-        const float lam = sm >= sp ? sm : sp;
+        T sm, sp;
+        const Quad<T> fm = quad_flux<DIR, true>(m, ph, &sm), fp = quad_flux<DIR, true>(p, ph, &sp);
+        const T lam = sm >= sp ? sm : sp;
         return qfma(qsub(m, p), lam, qadd(fm, fp));
     } else {
-        float a[4], b[4], F[4];
+        T a[4], b[4], F[4];
         qget(m, a);
         qget(p, b);
         roe_flux<DIR, true>(a, b, ph, F);
-        return qmul(qput(F), 2.f);
+        return qmul(qput(F), T(2));
     }
 }
 // F* - f from twice the common flux.
-__device__ __forceinline__ Quad half_jump(const Quad& G2, const Quad& f)
+template <class T>
+__device__ __forceinline__ Quad<T> half_jump(const Quad<T>& G2, const Quad<T>& f)
 {
-    return {pfma(G2.a, pbc(0.5f), pmul(f.a, pbc(-1.f))), pfma(G2.b, pbc(0.5f), pmul(f.b, pbc(-1.f)))};
+    return {pfma(G2.a, pbc(T(0.5)), pmul(f.a, pbc(T(-1)))), pfma(G2.b, pbc(T(0.5)), pmul(f.b, pbc(T(-1))))};
 }
 
 // x-line or y-line of one thread: derivative r, edge states lo, hi and edge
 // fluxes flo, fhi of the line x (consumed).
 template <int N, int DIR, int DIV>
-__device__ __forceinline__ void quad_line(const QuadTab& t, const Phys<float>& ph, Quad (&x)[N], Quad (&r)[N],
-                                          Quad& lo, Quad& hi, Quad& flo, Quad& fhi)
+__device__ __forceinline__ void quad_line(const QuadTab& t, const Phys<float>& ph, Quad<float> (&x)[N], Quad<float> (&r)[N],
+                                          Quad<float>& lo, Quad<float>& hi, Quad<float>& flo, Quad<float>& fhi)
 {
     lo = edge_lo<N>(t, x);
     hi = edge_hi<N>(t, x);
@@ -240,7 +249,7 @@ __device__ __forceinline__ void quad_line(const QuadTab& t, const Phys<float>& p
         fhi = edge_hi<N>(t, x);
         line_derivative<N>(t, x, r);
     } else {
-        Quad dq[N];
+        Quad<float> dq[N];
         line_derivative<N>(t, x, dq);
 #pragma unroll
         for (int a = 0; a < N; ++a) {
@@ -277,14 +286,14 @@ __device__ __forceinline__ void stage_tile_quad(const StageArgs<float>& A, const
     constexpr int N = P + 1, NN = N * N;
     constexpr int NT = TX * TY * N;
     using L = QuadLayout<N, TX, TY>;
-    Quad* sq = reinterpret_cast<Quad*>(smem_raw);
-    Quad* xR = sq + L::SQ;
-    Quad* xH = xR + L::XR;
-    Quad* xF = xH + L::XH;
-    Quad* yT = xF + L::XF;
-    Quad* yH = yT + L::YT;
-    Quad* yF = yH + L::YH;
-    Quad* avS = xR;  // row partial sums of the averages, over the edge states after phase 3
+    Quad<float>* sq = reinterpret_cast<Quad<float>*>(smem_raw);
+    Quad<float>* xR = sq + L::SQ;
+    Quad<float>* xH = xR + L::XR;
+    Quad<float>* xF = xH + L::XH;
+    Quad<float>* yT = xF + L::XF;
+    Quad<float>* yH = yT + L::YT;
+    Quad<float>* yF = yH + L::YH;
+    Quad<float>* avS = xR;  // row partial sums of the averages, over the edge states after phase 3
     static_assert(L::XR >= TX * TY * N, "the partial sums of the averages fit the right edge states");
 
     const int mode = MODE > 0 ? MODE : A.mode;
@@ -315,7 +324,7 @@ __device__ __forceinline__ void stage_tile_quad(const StageArgs<float>& A, const
 #pragma unroll
         for (int v = 0; v < 4; ++v) asm volatile("prefetch.global.L2 [%0];" ::"l"(A.lo + v * A.npts + e * NN));
     }
-    Quad x[N], rx[N], eL, fL;
+    Quad<float> x[N], rx[N], eL, fL;
     if (valid) load_row_quads<N>(A.qs, A.qb, addb, A.npts, off, x);
     {
         constexpr int NXH = 2 * TY * N, LINES = NXH + 2 * TX * N;
@@ -340,10 +349,10 @@ __device__ __forceinline__ void stage_tile_quad(const StageArgs<float>& A, const
             }
             if (have) {
                 const long long eh = ((long long)gj * A.nx + gi) * NN;
-                Quad h[N];
+                Quad<float> h[N];
                 if (xdir) load_row_quads<N>(A.qs, A.qb, addb, A.npts, eh + kk * N, h);
                 else load_col_quads<N>(A.qs, A.qb, addb, A.npts, eh + kk, h);
-                const Quad es = side ? edge_lo<N>(qt, h) : edge_hi<N>(qt, h);
+                const Quad<float> es = side ? edge_lo<N>(qt, h) : edge_hi<N>(qt, h);
                 if (xdir) {
                     if (side) xH[pos * N + kk] = es;
                     else xR[L::xr(pos, 0, kk)] = es;
@@ -357,7 +366,7 @@ __device__ __forceinline__ void stage_tile_quad(const StageArgs<float>& A, const
     if (valid) {
 #pragma unroll
         for (int a = 0; a < N; ++a) sq[L::sq(el, k, a)] = x[a];
-        Quad eR, fR;
+        Quad<float> eR, fR;
         quad_line<N, 0, DIV>(qt, A.ph, x, rx, eL, eR, fL, fR);
         xR[L::xr(ty, tx + 1, k)] = eR;
         xF[L::ef(el, k)] = fR;
@@ -375,9 +384,9 @@ __device__ __forceinline__ void stage_tile_quad(const StageArgs<float>& A, const
     const int txc = elc % TX, tyc = elc / TX;
     const bool validc = active && txc < TXe && tyc < TYe;
     const bool bwall = A.bcy && j0 + tyc == 0;
-    Quad ry[N], eB, gB;
+    Quad<float> ry[N], eB, gB;
     if (validc) {
-        Quad c[N], eT, gT;
+        Quad<float> c[N], eT, gT;
 #pragma unroll
         for (int b = 0; b < N; ++b) c[b] = sq[L::sq(elc, b, kc)];
         quad_line<N, 1, DIV>(qt, A.ph, c, ry, eB, eT, gB, gT);
@@ -390,23 +399,23 @@ __device__ __forceinline__ void stage_tile_quad(const StageArgs<float>& A, const
     if (validc) {
         // lower face: the jump F* - f of this element into its y-derivative,
         // the neighbour's over its top edge flux
-        const Quad dm = bwall ? eB : yT[L::yt(tyc, txc, kc)];
-        const Quad G = quad_face2<FLUX, 1>(dm, eB, A.ph);
-        const Quad J = half_jump(G, gB);
+        const Quad<float> dm = bwall ? eB : yT[L::yt(tyc, txc, kc)];
+        const Quad<float> G = quad_face2<FLUX, 1>(dm, eB, A.ph);
+        const Quad<float> J = half_jump(G, gB);
         if (tyc > 0) {
-            Quad* pj = yF + L::ef(elc - TX, kc);
+            Quad<float>* pj = yF + L::ef(elc - TX, kc);
             *pj = half_jump(G, *pj);
         }
 #pragma unroll
         for (int b = 0; b < N; ++b) sq[L::sq(elc, b, kc)] = qfma(J, qt.dgl[b], ry[b]);
     }
-    Quad JL;
+    Quad<float> JL;
     if (valid) {
-        const Quad dm = lwall ? eL : xR[L::xr(ty, tx, k)];
-        const Quad G = quad_face2<FLUX, 0>(dm, eL, A.ph);
+        const Quad<float> dm = lwall ? eL : xR[L::xr(ty, tx, k)];
+        const Quad<float> G = quad_face2<FLUX, 0>(dm, eL, A.ph);
         JL = half_jump(G, fL);
         if (tx > 0) {
-            Quad* pj = xF + L::ef(el - 1, k);
+            Quad<float>* pj = xF + L::ef(el - 1, k);
             *pj = half_jump(G, *pj);
         }
     }
@@ -417,10 +426,10 @@ __device__ __forceinline__ void stage_tile_quad(const StageArgs<float>& A, const
         const int pos = r / N, kk = r % N;
         if (pos < (xe ? TYe : TXe)) {
             const bool wall = xe ? (A.bcx && i0 + TXe == A.nx) : (A.bcy && j0 + TYe == A.ny);
-            const Quad Em = xe ? xR[L::xr(pos, TXe, kk)] : yT[L::yt(TYe, pos, kk)];
-            const Quad dp = wall ? Em : (xe ? xH[pos * N + kk] : yH[pos * N + kk]);
-            const Quad G = xe ? quad_face2<FLUX, 0>(Em, dp, A.ph) : quad_face2<FLUX, 1>(Em, dp, A.ph);
-            Quad* pj = xe ? xF + L::ef(pos * TX + TXe - 1, kk) : yF + L::ef((TYe - 1) * TX + pos, kk);
+            const Quad<float> Em = xe ? xR[L::xr(pos, TXe, kk)] : yT[L::yt(TYe, pos, kk)];
+            const Quad<float> dp = wall ? Em : (xe ? xH[pos * N + kk] : yH[pos * N + kk]);
+            const Quad<float> G = xe ? quad_face2<FLUX, 0>(Em, dp, A.ph) : quad_face2<FLUX, 1>(Em, dp, A.ph);
+            Quad<float>* pj = xe ? xF + L::ef(pos * TX + TXe - 1, kk) : yF + L::ef((TYe - 1) * TX + pos, kk);
             *pj = half_jump(G, *pj);
         }
     }
@@ -440,12 +449,12 @@ __device__ __forceinline__ void stage_tile_quad(const StageArgs<float>& A, const
         if (mode == MODE_INC2) w *= 0.25f;
         if (mode == MODE_INC3) w *= 2.0f / 3.0f;
         const float sx = -A.rhx2 * w, sy = -A.rhy2 * w;
-        const Quad JR = xF[L::ef(el, k)];
+        const Quad<float> JR = xF[L::ef(el, k)];
 #pragma unroll
         for (int a = 0; a < N; ++a) {
-            Quad y = sq[L::sq(el, k, a)];
+            Quad<float> y = sq[L::sq(el, k, a)];
             y = qfma(yF[L::ef(el, a)], grk, y);
-            Quad z = qfma(JL, qt.dgl[a], rx[a]);
+            Quad<float> z = qfma(JL, qt.dgl[a], rx[a]);
             z = qfma(JR, -qt.dgl[N - 1 - a], z);
             float yv[4], zv[4];
             qget(qmul(y, sy), yv);
@@ -506,7 +515,7 @@ __device__ __forceinline__ void stage_tile_quad(const StageArgs<float>& A, const
         __syncthreads();
         const int ax = tid % TX, ay = tid / TX;
         if (tid < TX * TY && ax < TXe && ay < TYe) {
-            Quad s = avS[L::ef(tid, 0)];
+            Quad<float> s = avS[L::ef(tid, 0)];
 #pragma unroll
             for (int b = 1; b < N; ++b) s = qadd(s, avS[L::ef(tid, b)]);
             float sv[4];
