@@ -633,15 +633,22 @@ struct TabPr {
 
 // Operator tables of the quad form (cpr_stage_quad.cuh), which uses the
 // symmetry of the solution points: lm[l] = l_l(-1) = l_{N-1-l}(+1); dgl[a] =
-// g_L'(xi_a) = -g_R'(xi_{N-1-a}); and the derivative as a combination of the
-// N - 1 differences f_{m+1} - f_m, f'_a = sum_m C_am (f_{m+1} - f_m), with C_am
-// = sum_{l > m} D_al = C_{N-1-a,N-2-m}, split over mirrored differences:
-// ce = (C_am + C_a,N-2-m) / 2, co = (C_am - C_a,N-2-m) / 2, cm the middle
-// difference's (even N).
+// g_L'(xi_a) = -g_R'(xi_{N-1-a}); and a line operator D (the derivative, or the
+// joined one of line_derivative) as a combination of the N - 1 differences
+// f_{m+1} - f_m, sum_m C_am (f_{m+1} - f_m), with C_am = sum_{l > m} D_al =
+// C_{N-1-a,N-2-m}, split over mirrored differences: ce = (C_am + C_a,N-2-m) / 2,
+// co = (C_am - C_a,N-2-m) / 2, cm the middle difference's (even N).
+template <class T>
 struct QuadTab {
-    float lm[kMaxN], dgl[kMaxN];
-    float ce[(kMaxN + 1) / 2][2], co[(kMaxN + 1) / 2][2], cm[(kMaxN + 1) / 2];
+    T lm[kMaxN], dgl[kMaxN];
+    T ce[(kMaxN + 1) / 2][2], co[(kMaxN + 1) / 2][2], cm[(kMaxN + 1) / 2];
 };
+// The LP divergence takes the joined operator.
+template <class T>
+__host__ __device__ constexpr bool quad_joined(int n)
+{
+    return n >= 4;
+}
 
 // Unsigned division by an invariant divisor d (Granlund & Montgomery,
 // "Division by Invariant Integers using Multiplication", 1994): with

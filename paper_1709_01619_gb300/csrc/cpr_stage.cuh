@@ -54,7 +54,7 @@ template <class T>
 struct QuadArgs {};
 template <>
 struct QuadArgs<float> {
-    QuadTab tab;
+    QuadTab<float> tab;
     unsigned int tx_magic;
     int tx_shift;
 };

@@ -181,7 +181,7 @@ static StageArgs<T> make_stage_args(const LaunchCfg& c, int mode, const StagePtr
     A.tab = host_tab<T>(c.tab);
     A.tp = host_tabpr<T>(c.tab);
     if constexpr (sizeof(T) == 4) {
-        A.qx.tab = host_quadtab(c.tab);
+        A.qx.tab = host_quadtab<float>(c.tab, c.div == DIV_LP && quad_joined<float>(c.p + 1));
         div_magic((unsigned)A.tiles_x, &A.qx.tx_magic, &A.qx.tx_shift);
     }
     return A;

@@ -49,49 +49,72 @@ __device__ __forceinline__ void qget(const Quad<T>& x, T* v)
 template <class T>
 __device__ __forceinline__ Quad<T> qput(const T* v) { return qmk(v[0], v[1], v[2], v[3]); }
 
-// Edge states of a line of N quads at -1 (lo) and +1 (hi).  The solution
+// The same on a single variable.
+template <class T>
+__device__ __forceinline__ T qmul(T x, T c) { return c * x; }
+template <class T>
+__device__ __forceinline__ T qfma(T x, T c, T y) { return fma(c, x, y); }
+template <class T>
+__device__ __forceinline__ T qadd(T x, T y) { return x + y; }
+template <class T>
+__device__ __forceinline__ T qsub(T x, T y) { return x - y; }
+
+// Edge states of a line of N quads (or of N values of one variable) at -1 (lo) and +1 (hi).  The solution
 // points are symmetric, so l_l(+1) = l_{N-1-l}(-1): one table serves both.
 // Every edge state of the kernel, the element's own and the one a neighbour
 // CTA forms from its halo line, is one of these two sums in this order.
-template <int N>
-__device__ __forceinline__ Quad<float> edge_lo(const QuadTab& t, const Quad<float> (&x)[N])
+template <int N, class T, class X>
+__device__ __forceinline__ X edge_lo(const QuadTab<T>& t, const X (&x)[N])
 {
-    Quad<float> s = qmul(x[0], t.lm[0]);
+    X s = qmul(x[0], t.lm[0]);
 #pragma unroll
     for (int l = 1; l < N; ++l) s = qfma(x[l], t.lm[l], s);
     return s;
 }
-template <int N>
-__device__ __forceinline__ Quad<float> edge_hi(const QuadTab& t, const Quad<float> (&x)[N])
+template <int N, class T, class X>
+__device__ __forceinline__ X edge_hi(const QuadTab<T>& t, const X (&x)[N])
 {
-    Quad<float> s = qmul(x[N - 1], t.lm[0]);
+    X s = qmul(x[N - 1], t.lm[0]);
 #pragma unroll
     for (int l = 1; l < N; ++l) s = qfma(x[N - 1 - l], t.lm[l], s);
     return s;
 }
 
-// Derivative of the interpolant of a line at its N points.  The rows of D sum
-// to zero, so it is a combination of the N - 1 differences of neighbouring
-// values (exact for values within a factor of two, where the plain row sum
-// rounds every product of an O(1) value); and D changes sign under the mirror
-// image of the line, so sums and differences of mirrored differences serve
-// two points at once: 8 / 13 / 22 operations per pair of variables for
-// N = 3 / 4 / 5 against 9 / 16 / 25 of the row sums.
-template <int N>
-__device__ __forceinline__ void line_derivative(const QuadTab& t, const Quad<float> (&f)[N], Quad<float> (&r)[N])
+// A line operator with the mirror symmetry of the points applied to a line:
+// the derivative of the interpolant, or the one of the LP divergence below.
+// Its rows sum to zero, so it is a combination of the N - 1 differences of
+// neighbouring values (exact for values within a factor of two, where the
+// plain row sum rounds every product of an O(1) value); and it changes sign
+// under the mirror image of the line, so sums and differences of mirrored
+// differences serve two points at once: 8 / 13 / 22 operations per pair of
+// variables for N = 3 / 4 / 5 against 9 / 16 / 25 of the row sums.
+//
+// LP divergence: sum_l D_al f_l + (F*_L - f_L) g_L'_a + (F*_R - f_R) g_R'_a with
+// the interpolated edge fluxes f_L = sum_l l_l(-1) f_l, f_R likewise.  Written
+// with f_0 and f_{N-1} in place of f_L and f_R, the rest of the edge terms
+// joins the matrix,
+//   D'_al = D_al + (delta_l0 - l_l(-1)) g_L'_a + (delta_l,N-1 - l_l(+1)) g_R'_a,
+// which keeps both properties (the l(+-1) sum to one).  So no edge flux is
+// interpolated, N / 2 operations per point and pair of variables, and their
+// rounding is gone.  FP32 with N >= 4 (1024^2 p = 3 4.50 -> 4.46 ms for 8 steps,
+// 128^2 1.115 -> 1.104 ms for 64; error against 64 bits 5.3e-8 -> 4.5e-8 and
+// 1.1e-7 -> 9e-8); for N = 3, where the registers are full, it spills (1365 x
+// 1363 4.73 -> 4.77 ms).
+template <int N, class T, class X>
+__device__ __forceinline__ void line_derivative(const QuadTab<T>& t, const X (&f)[N], X (&r)[N])
 {
     constexpr int M = N - 1, H = M / 2;
-    Quad<float> s[H > 0 ? H : 1], d[H > 0 ? H : 1], mid;
+    X s[H > 0 ? H : 1], d[H > 0 ? H : 1], mid;
 #pragma unroll
     for (int m = 0; m < H; ++m) {
-        const Quad<float> lo = qsub(f[m + 1], f[m]), hi = qsub(f[N - 1 - m], f[N - 2 - m]);
+        const X lo = qsub(f[m + 1], f[m]), hi = qsub(f[N - 1 - m], f[N - 2 - m]);
         s[m] = qadd(lo, hi);
         d[m] = qsub(lo, hi);
     }
     if constexpr (M % 2 == 1) mid = qsub(f[H + 1], f[H]);
 #pragma unroll
     for (int a = 0; a < (N + 1) / 2; ++a) {
-        Quad<float> p;
+        X p;
         if constexpr (M % 2 == 1) {
             p = qmul(mid, t.cm[a]);
 #pragma unroll
@@ -104,7 +127,7 @@ __device__ __forceinline__ void line_derivative(const QuadTab& t, const Quad<flo
         if (2 * a == N - 1) {
             r[a] = p;
         } else {
-            Quad<float> lo = p, hi = p;
+            X lo = p, hi = p;
 #pragma unroll
             for (int m = 0; m < H; ++m) {
                 lo = qfma(d[m], t.co[a][m], lo);
@@ -234,10 +257,12 @@ __device__ __forceinline__ Quad<T> half_jump(const Quad<T>& G2, const Quad<T>& f
     return {pfma(G2.a, pbc(T(0.5)), pmul(f.a, pbc(T(-1)))), pfma(G2.b, pbc(T(0.5)), pmul(f.b, pbc(T(-1))))};
 }
 
-// x-line or y-line of one thread: derivative r, edge states lo, hi and edge
-// fluxes flo, fhi of the line x (consumed).
+// x-line or y-line of one thread: line operator r, edge states lo, hi and the
+// fluxes flo, fhi that the common fluxes are compared with (joined operator:
+// those of the first and last point; else of the edges) of the line x
+// (consumed).
 template <int N, int DIR, int DIV>
-__device__ __forceinline__ void quad_line(const QuadTab& t, const Phys<float>& ph, Quad<float> (&x)[N], Quad<float> (&r)[N],
+__device__ __forceinline__ void quad_line(const QuadTab<float>& t, const Phys<float>& ph, Quad<float> (&x)[N], Quad<float> (&r)[N],
                                           Quad<float>& lo, Quad<float>& hi, Quad<float>& flo, Quad<float>& fhi)
 {
     lo = edge_lo<N>(t, x);
@@ -245,8 +270,13 @@ __device__ __forceinline__ void quad_line(const QuadTab& t, const Phys<float>& p
     if constexpr (DIV == DIV_LP) {
 #pragma unroll
         for (int a = 0; a < N; ++a) x[a] = quad_flux<DIR>(x[a], ph);
-        flo = edge_lo<N>(t, x);
-        fhi = edge_hi<N>(t, x);
+        if constexpr (quad_joined<float>(N)) {
+            flo = x[0];
+            fhi = x[N - 1];
+        } else {
+            flo = edge_lo<N>(t, x);
+            fhi = edge_hi<N>(t, x);
+        }
         line_derivative<N>(t, x, r);
     } else {
         Quad<float> dq[N];
@@ -303,7 +333,7 @@ __device__ __forceinline__ void stage_tile_quad(const StageArgs<float>& A, const
     if (A.do_avg && tile == 0 && tid == 0) A.ctrl->marked = 0;
 
     const bool active = tid < NT;
-    const QuadTab& qt = qx.tab;
+    const QuadTab<float>& qt = qx.tab;
     const int tj = (int)div_invariant((unsigned)tile, (unsigned)A.tiles_x, A.qx.tx_magic, A.qx.tx_shift);
     const int i0 = (tile - tj * A.tiles_x) * TX;
     const int j0 = tj * TY;

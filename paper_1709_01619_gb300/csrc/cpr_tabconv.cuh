@@ -50,26 +50,33 @@ inline TabPr<T> host_tabpr(const HostTab& h)
     return t;
 }
 
-// The tables of the quad form (QuadTab), formed in FP64.
-inline QuadTab host_quadtab(const HostTab& h)
+// The tables of the quad form (QuadTab), formed in FP64.  joined: the operator
+// D' of line_derivative (LP divergence), else D.
+template <class T>
+inline QuadTab<T> host_quadtab(const HostTab& h, bool joined)
 {
-    QuadTab t{};
+    QuadTab<T> t{};
     const int n = h.n;
     for (int a = 0; a < n; ++a) {
-        t.lm[a] = float(h.lm[a]);
-        t.dgl[a] = float(h.dgl[a]);
+        t.lm[a] = T(h.lm[a]);
+        t.dgl[a] = T(h.dgl[a]);
     }
     for (int a = 0; a < (n + 1) / 2; ++a) {
+        auto at = [&](int l) {
+            double d = h.D[a][l];
+            if (joined) d += ((l == 0) - h.lm[l]) * h.dgl[a] + ((l == n - 1) - h.lp[l]) * h.dgr[a];
+            return d;
+        };
         auto C = [&](int m) {
             double s = 0.0;
-            for (int l = n - 1; l > m; --l) s += h.D[a][l];
+            for (int l = n - 1; l > m; --l) s += at(l);
             return s;
         };
         for (int m = 0; m < (n - 1) / 2; ++m) {
-            t.ce[a][m] = float(0.5 * (C(m) + C(n - 2 - m)));
-            t.co[a][m] = float(0.5 * (C(m) - C(n - 2 - m)));
+            t.ce[a][m] = T(0.5 * (C(m) + C(n - 2 - m)));
+            t.co[a][m] = T(0.5 * (C(m) - C(n - 2 - m)));
         }
-        if (n % 2 == 0) t.cm[a] = float(C(n / 2 - 1));
+        if (n % 2 == 0) t.cm[a] = T(C(n / 2 - 1));
     }
     return t;
 }
