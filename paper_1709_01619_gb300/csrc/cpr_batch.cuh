@@ -50,7 +50,7 @@ struct BatchArgs {
     int swap;          // increment form: the high part of q^n is in Y (else X)
     Tab<T> tab;        // operator tables of the group's order
     TabPr<T> tp;       // the same in pairs over points
-    QuadArgs<T> qx;    // the tables of the quad form (FP32 Euler)
+    QuadArgs<T> qx;    // the tables of the quad forms (Euler)
 };
 
 // Register budget: as the single-problem kernel.
@@ -77,10 +77,8 @@ __device__ __forceinline__ void batch_item(const BatchArgs<T>& B, int w, StageAr
         A.bcx = I.bcx;
         A.bcy = I.bcy;
         A.tiles_x = I.tiles_x;
-        if constexpr (sizeof(T) == 4) {
-            A.qx.tx_magic = I.tx_magic;
-            A.qx.tx_shift = I.tx_shift;
-        }
+        A.qx.tx_magic = I.tx_magic;
+        A.qx.tx_shift = I.tx_shift;
         A.mode = B.mode;
         A.do_avg = 0;
         A.avg = nullptr;
@@ -107,7 +105,9 @@ __device__ __forceinline__ void batch_item(const BatchArgs<T>& B, int w, StageAr
         s_n = I.ntiles;
     }
     __syncthreads();
-    if constexpr (stage_quad<T, EQ, DELTA>)
+    if constexpr (sizeof(T) == 8 && EQ == EQ_EULER)
+        stage_tile_f64<P, DIV, FLUX, TX, TY>(sA, B.tab, B.qx, s_t, threadIdx.x, smem_raw, s_n);
+    else if constexpr (stage_quad<T, EQ, DELTA>)
         stage_tile_quad<P, DIV, FLUX, TX, TY, false, 0>(sA, B.tab, B.qx, s_t, threadIdx.x, smem_raw, s_n);
     else
         stage_tile<T, P, EQ, DIV, FLUX, TX, TY, DELTA>(sA, B.tab, B.tp, s_t, threadIdx.x, smem_raw, s_n);
@@ -117,10 +117,10 @@ __device__ __forceinline__ void batch_item(const BatchArgs<T>& B, int w, StageAr
 // has one CTA per work item.  The loop costs registers (the tile body spills
 // more inside it), so the autotuner weighs both forms.
 template <class T, int P, int EQ, int DIV, int FLUX, int TX, int TY, bool DELTA, bool PERSIST>
-__global__ void __launch_bounds__(TX * TY * (P + 1), (batch_min_blocks<T, P + 1>()))
+__global__ void __launch_bounds__((stage_block<T, P, EQ, TX, TY>), (batch_min_blocks<T, P + 1>()))
 cpr_batch_stage_kernel(const BatchArgs<T> B)
 {
-    static_assert((TX * TY * (P + 1)) % 32 == 0, "whole warps: the warp-level reductions use every lane");
+    static_assert(stage_block<T, P, EQ, TX, TY> % 32 == 0, "whole warps: the warp-level reductions use every lane");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     // The work item's arguments live in shared memory, read at their points
     // of use instead of occupying registers through the whole tile.

@@ -10,9 +10,8 @@ namespace cpr {
 template <class T, int P, int EQ, int FLUX, int FAM>
 static cudaError_t batch_one(const BatchArgs<T>& B, int grid, cudaStream_t s, int what, int* occ)
 {
-    constexpr int N = P + 1;
     constexpr int TX = BatchTile<FAM>::X, TY = BatchTile<FAM>::Y;
-    constexpr int NT = TX * TY * N;
+    constexpr int NT = stage_block<T, P, EQ, TX, TY>;
     auto loop = cpr_batch_stage_kernel<T, P, EQ, DIV_LP, FLUX, TX, TY, stage_delta<T>(), true>;
     auto flat = cpr_batch_stage_kernel<T, P, EQ, DIV_LP, FLUX, TX, TY, stage_delta<T>(), false>;
     const size_t smem = stage_smem<T, P, EQ, TX, TY, stage_delta<T>()>();

@@ -103,16 +103,42 @@ __device__ __forceinline__ float fsqrt_ftz(float x)
     asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
+// In FP64, where an operation keeps a scheduler busy for 64 cycles: the ~20-bit
+// hardware seed y and one third-order correction from the residual e, the
+// binomial series of (1 - e)^-1 and (1 - e)^-1/2 cut after e^2 (Householder's
+// method of order 2; the next term is below 2^-57):
+//   1/x = y (1 + e + e^2), e = 1 - x y;
+//   sqrt(x) = s (1 + e/2 + 3 e^2/8), s = x y, e = 1 - s y.
+// Three and five operations.  Zeros, infinities and NaN keep the IEEE results
+// (tested on the bits, off the FP64 pipe); subnormal operands count as zero.
+__device__ __forceinline__ double frcp_ftz(double x)
+{
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x, y, 1.0);
+    const double r = fma(y, fma(e, e, e), y);
+    const unsigned int h = (unsigned int)__double2hiint(x) & 0x7fffffffu;
+    return h - 0x00100000u < 0x7fe00000u ? r : y;
+}
+__device__ __forceinline__ double fsqrt_ftz(double x)
+{
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double s = x * y, e = fma(-s, y, 1.0);
+    const double r = fma(s, fma(0.375, e, 0.5) * e, s);
+    const unsigned int h = (unsigned int)__double2hiint(x);
+    return h - 0x00100000u >= 0x7fe00000u && h <= 0x80000000u ? x : r;
+}
 template <bool FTZ, class T>
 __device__ __forceinline__ T rcp_of(T x)
 {
-    if constexpr (FTZ && sizeof(T) == 4) return frcp_ftz(x);
+    if constexpr (FTZ) return frcp_ftz(x);
     else return frcp(x);
 }
 template <bool FTZ, class T>
 __device__ __forceinline__ T sqrt_of(T x)
 {
-    if constexpr (FTZ && sizeof(T) == 4) return fsqrt_ftz(x);
+    if constexpr (FTZ) return fsqrt_ftz(x);
     else return fsqrt(x);
 }
 
@@ -124,7 +150,10 @@ __device__ __forceinline__ T pressure(const T* q, T gamma, T& u, T& v, T& r)
     r = rcp_of<FTZ>(q[0]);
     u = q[1] * r;
     v = q[2] * r;
-    return (gamma - T(1)) * (q[3] - T(0.5) * (q[1] * u + q[2] * v));
+    // FP64: the fused operations written out, so that every kernel that holds
+    // this point rounds alike
+    if constexpr (sizeof(T) == 8) return (gamma - T(1)) * fma(T(-0.5), fma(q[1], u, q[2] * v), q[3]);
+    else return (gamma - T(1)) * (q[3] - T(0.5) * (q[1] * u + q[2] * v));
 }
 template <class T>
 __device__ __forceinline__ T pressure(const T* q, T gamma, T& u, T& v)
@@ -302,7 +331,7 @@ __device__ __forceinline__ T point_speed(const T* q, const Phys<T>& ph)
     } else {
         T u, v, r;
         T p = pressure<FTZ>(q, ph.gamma, u, v, r);
-        return sqrt_of<FTZ>(u * u + v * v) + sqrt_of<FTZ>(ph.gamma * p * r);
+        return sqrt_of<FTZ>(fma(u, u, v * v)) + sqrt_of<FTZ>(ph.gamma * p * r);
     }
 }
 
@@ -643,11 +672,11 @@ struct QuadTab {
     T lm[kMaxN], dgl[kMaxN];
     T ce[(kMaxN + 1) / 2][2], co[(kMaxN + 1) / 2][2], cm[(kMaxN + 1) / 2];
 };
-// The LP divergence takes the joined operator.
+// The LP divergence takes the joined operator (in FP64 for every order).
 template <class T>
 __host__ __device__ constexpr bool quad_joined(int n)
 {
-    return n >= 4;
+    return sizeof(T) == 8 || n >= 4;
 }
 
 // Unsigned division by an invariant divisor d (Granlund & Montgomery,

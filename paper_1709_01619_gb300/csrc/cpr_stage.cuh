@@ -48,13 +48,11 @@
 
 namespace cpr {
 
-// What only the quad form (FP32 Euler) needs: its tables and the division of
-// a tile index by tiles_x (div_invariant).  Nothing for FP64.
+// What only the quad forms (Euler) need: their tables and the division of a
+// tile index by tiles_x (div_invariant).
 template <class T>
-struct QuadArgs {};
-template <>
-struct QuadArgs<float> {
-    QuadTab<float> tab;
+struct QuadArgs {
+    QuadTab<T> tab;
     unsigned int tx_magic;
     int tx_shift;
 };
@@ -79,7 +77,7 @@ struct StageArgs {
     Phys<T> ph;
     Tab<T> tab;
     TabPr<T> tp;      // the tables in pairs over points (two-lane path)
-    QuadArgs<T> qx;   // the quad form's own arguments (FP32 Euler)
+    QuadArgs<T> qx;   // the quad forms' own arguments (Euler)
 };
 
 template <int N, int V, int TX, int TY, bool DELTA>
@@ -341,12 +339,6 @@ constexpr bool stage_delta()
 // compiled for two resident CTAs: twice the registers let the compiler keep
 // more loads in flight, which is what bounds a CTA when the SM holds only
 // one or two of them.
-// FP64 p = 3: two resident CTAs (124 registers, no spills; one CTA of 134
-// registers left the 128 x 128 grid two waves deep: 76.2 -> 73.8 ms for 200
-// steps); the other FP64 orders already fit two.
-#ifndef CPR_STAGE_MINB_FP64_N4
-#define CPR_STAGE_MINB_FP64_N4 2
-#endif
 #ifndef CPR_STAGE_MINB_WIDE
 #define CPR_STAGE_MINB_WIDE 2
 #endif
@@ -358,15 +350,19 @@ constexpr int stage_min_blocks()
 {
     static_assert(64 % ELEMS == 0, "tiles of 64 elements or a divisor of it");
     return (64 / ELEMS) *
-           (sizeof(T) == 8 ? (N == 4 ? CPR_STAGE_MINB_FP64_N4 : 1)
+           (sizeof(T) == 8 ? 1
             : WIDE         ? CPR_STAGE_MINB_WIDE
                            : (N == 2 ? CPR_STAGE_MINB_FP32_N2
                                      : (N == 3 ? CPR_STAGE_MINB_FP32_N3
                                                : (N == 4 ? CPR_STAGE_MINB_FP32 : CPR_STAGE_MINB_FP32_N5))));
 }
 
+// Threads of a CTA: whole warps (the warp-level reductions use every lane).
+constexpr int stage_threads(int n) { return (n + 31) / 32 * 32; }
+
 }  // namespace cpr
 
+#include "cpr_stage_f64.cuh"
 #include "cpr_stage_quad.cuh"
 
 namespace cpr {
@@ -380,9 +376,14 @@ constexpr bool stage_quad = sizeof(T) == 4 && EQ == EQ_EULER && !DELTA;
 template <class T, int P, int EQ, int TX, int TY, bool DELTA>
 constexpr size_t stage_smem()
 {
-    if constexpr (stage_quad<T, EQ, DELTA>) return sizeof(Quad<float>) * QuadLayout<P + 1, TX, TY>::TOTAL;
+    if constexpr (sizeof(T) == 8 && EQ == EQ_EULER) return sizeof(Quad<double>) * F64Layout<P + 1, TX, TY>::TOTAL;
+    else if constexpr (stage_quad<T, EQ, DELTA>) return sizeof(Quad<float>) * QuadLayout<P + 1, TX, TY>::TOTAL;
     else return sizeof(T) * StageLayout<P + 1, NVars<EQ>::value, TX, TY, DELTA>::TOTAL;
 }
+
+// Threads of a stage-update CTA.
+template <class T, int P, int EQ, int TX, int TY>
+constexpr int stage_block = sizeof(T) == 8 && EQ == EQ_EULER ? 2 * f64_role_threads(P, TX, TY) : TX * TY * (P + 1);
 
 // One tile of the stage: the work of one CTA.  tile indexes the instance's
 // TX x TY tiles (row-major); threads tid >= NT of a wider CTA only take part

@@ -10,12 +10,6 @@
 #include "cpr_stage.cuh"
 #include "cpr_adjoint.cuh"
 
-// Small-tile FP64 stage kernel for grids of at most one tile per two SMs
-// (0: off).
-#ifndef CPR_STAGE_SMALL
-#define CPR_STAGE_SMALL 1
-#endif
-
 namespace cpr {
 
 
@@ -53,9 +47,56 @@ static cudaError_t with_quad_kernel(int mode, bool wide, bool shared, F&& f)
     }
 }
 
+// The tile of a single FP64 problem.  A stage takes the time of the scheduler
+// with most warps (cpr_stage_f64.cuh): of the tiles, the one with the fewest
+// warps on the busiest scheduler, each step down counted 10 % dearer for its
+// longer boundary.  An instance of a batch (sms 0) takes the largest.
+// us per Euler stage, p = 3: 16^2 elements 16.7 (4 x 4), 64^2 26.4, 96^2 45.9
+// (8 x 8 tiles, one thread for a row and a column: 36 at every size below 64^2).
+inline int f64_tile(const LaunchCfg& c)
+{
+    int best = 0;
+    double cost = 0.0, dearer = 1.0;
+    for (int k = 0; c.sms > 0 && k < f64_tiles(c.p); ++k, dearer *= 1.1) {
+        const int tx = f64_tile_x(k), ty = f64_tile_y(k);
+        const long long ctas = (long long)((c.nx + tx - 1) / tx) * ((c.ny + ty - 1) / ty);
+        const long long warps = (ctas + c.sms - 1) / c.sms * (2 * f64_role_threads(c.p, tx, ty) / 32);
+        const double w = (double)((warps + 3) / 4) * dearer;
+        if (k == 0 || w < cost) {
+            best = k;
+            cost = w;
+        }
+    }
+    return best;
+}
+
+template <int P, int DIV, int FLUX, int K>
+static cudaError_t stage_f64_tile(const LaunchCfg& c, StageArgs<double> A, cudaStream_t s, bool prep)
+{
+    constexpr int TX = f64_tile_x(K), TY = f64_tile_y(K);
+    const size_t smem = stage_smem<double, P, EQ_EULER, TX, TY, false>();
+    auto kern = cpr_stage_f64_kernel<P, DIV, FLUX, TX, TY, f64_min_blocks(P, K)>;
+    if (prep) return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    A.tiles_x = (c.nx + TX - 1) / TX;
+    div_magic((unsigned)A.tiles_x, &A.qx.tx_magic, &A.qx.tx_shift);
+    kern<<<A.tiles_x * ((c.ny + TY - 1) / TY), 2 * f64_role_threads(P, TX, TY), smem, s>>>(A);
+    return cudaGetLastError();
+}
+
+template <int P, int DIV, int FLUX>
+static cudaError_t stage_f64(const LaunchCfg& c, const StageArgs<double>& A, cudaStream_t s, bool prep)
+{
+    const int k = f64_tile(c);
+    if constexpr (f64_tiles(P) > 2)
+        if (k == 2) return stage_f64_tile<P, DIV, FLUX, 2>(c, A, s, prep);
+    return k == 1 ? stage_f64_tile<P, DIV, FLUX, 1>(c, A, s, prep) : stage_f64_tile<P, DIV, FLUX, 0>(c, A, s, prep);
+}
+
 template <class T, int P, int EQ, int DIV, int FLUX>
 static cudaError_t stage_one(const LaunchCfg& c, const StageArgs<T>& A, int ctas, cudaStream_t s, bool prep)
 {
+    if constexpr (sizeof(T) == 8 && EQ == EQ_EULER) return stage_f64<P, DIV, FLUX>(c, A, s, prep);
+    else {
     constexpr int N = P + 1, V = NVars<EQ>::value;
     constexpr int TX = stage_tile_x(P), TY = stage_tile_y(P);
     constexpr int NT = TX * TY * N;
@@ -78,17 +119,6 @@ static cudaError_t stage_one(const LaunchCfg& c, const StageArgs<T>& A, int ctas
     // device at once up to that many per SM
     constexpr int WIDE_PER_SM = stage_min_blocks<T, N, true, TX * TY>();
     const bool wide = HAS_WIDE && c.sms > 0 && ctas <= WIDE_PER_SM * c.sms;
-    // and, in FP64, tiles of 4 x 4 elements for grids of at most one tile per
-    // two SMs: four times the CTAs, so that more SMs share the FP64 work of a
-    // grid that would leave most of them idle (Euler, LP divergence, Rusanov
-    // flux; 24^2 p = 3 192.6 -> 109.9 ms for 1003 steps, 64^2 514 -> 317 ms;
-    // at 96^2, 144 tiles, slower: 773 -> 807 ms; in FP32 slower at every size,
-    // 24^2 17.1 -> 17.5 ms, 96^2 70.5 -> 78.9 ms)
-    // (whole warps only: p = 1 and 3, 32 and 64 threads)
-    constexpr int SX = 4, SY = 4;
-    constexpr bool HAS_SMALL = sizeof(T) == 8 && EQ == EQ_EULER && DIV == DIV_LP && FLUX == FLUX_RUSANOV &&
-                               (SX * SY * N) % 32 == 0 && CPR_STAGE_SMALL != 0;
-    [[maybe_unused]] const size_t smem_s = sizeof(T) * StageLayout<N, V, SX, SY, DELTA>::TOTAL;
     if (prep) {
         auto limit = [](auto k, size_t bytes) {
             return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
@@ -96,9 +126,6 @@ static cudaError_t stage_one(const LaunchCfg& c, const StageArgs<T>& A, int ctas
         cudaError_t e = limit(kern, smem);
         if (e == cudaSuccess && HAS_PF) e = limit(kern_pf, QUAD ? smem_q : smem);
         if (e == cudaSuccess && HAS_WIDE) e = limit(kern_w, smem);
-        if constexpr (HAS_SMALL)
-            if (e == cudaSuccess)
-                e = limit(cpr_stage_kernel<T, P, EQ, DIV, FLUX, SX, SY, DELTA, false, true>, smem_s);
         if constexpr (QUAD)
             for (int mode = MODE_SO1; mode <= MODE_INC3 && e == cudaSuccess; ++mode) {
                 auto lq = [&](auto k) { return limit(k, smem_q); };
@@ -106,16 +133,6 @@ static cudaError_t stage_one(const LaunchCfg& c, const StageArgs<T>& A, int ctas
                 if (e == cudaSuccess) e = with_quad_kernel<P, DIV, FLUX, TX, TY>(mode, true, c.shared, lq);
             }
         return e;
-    }
-    if constexpr (HAS_SMALL) {
-        if (c.sms > 0 && 2 * ctas <= c.sms) {
-            StageArgs<T> As = A;
-            As.tiles_x = (c.nx + SX - 1) / SX;
-            const int grid = As.tiles_x * ((c.ny + SY - 1) / SY);
-            cpr_stage_kernel<T, P, EQ, DIV, FLUX, SX, SY, DELTA, false, true>
-                <<<grid, SX * SY * N, smem_s, s>>>(As);
-            return cudaGetLastError();
-        }
     }
     if constexpr (QUAD) {
         if (A.mode != MODE_RESIDUAL) {
@@ -127,10 +144,10 @@ static cudaError_t stage_one(const LaunchCfg& c, const StageArgs<T>& A, int ctas
             return with_quad_kernel<P, DIV, FLUX, TX, TY>(A.mode, wide, c.shared, launch);
         }
     }
-    if (HAS_PF && A.pf_lo) kern_pf<<<ctas, NT, smem, s>>>(A);
-    else if (wide) kern_w<<<ctas, NT, smem, s>>>(A);
+    if (wide) kern_w<<<ctas, NT, smem, s>>>(A);
     else kern<<<ctas, NT, smem, s>>>(A);
     return cudaGetLastError();
+    }
 }
 
 template <class T, int P>
@@ -180,10 +197,8 @@ static StageArgs<T> make_stage_args(const LaunchCfg& c, int mode, const StagePtr
     A.ph.ay = T(c.ay);
     A.tab = host_tab<T>(c.tab);
     A.tp = host_tabpr<T>(c.tab);
-    if constexpr (sizeof(T) == 4) {
-        A.qx.tab = host_quadtab<float>(c.tab, c.div == DIV_LP && quad_joined<float>(c.p + 1));
-        div_magic((unsigned)A.tiles_x, &A.qx.tx_magic, &A.qx.tx_shift);
-    }
+    A.qx.tab = host_quadtab<T>(c.tab, c.div == DIV_LP && quad_joined<T>(c.p + 1));
+    div_magic((unsigned)A.tiles_x, &A.qx.tx_magic, &A.qx.tx_shift);
     return A;
 }
 

@@ -139,6 +139,29 @@ __device__ __forceinline__ void line_derivative(const QuadTab<T>& t, const X (&f
     }
 }
 
+// S quads in shared memory.  Every access is of 16 bytes: a whole FP32 quad,
+// or one of the two pairs of an FP64 quad, which lie in planes of their own so
+// that both types meet the same banks.
+template <class T, int S>
+struct QuadArr {
+    Pr<T>* p;
+    __device__ __forceinline__ Quad<T> ld(int i) const
+    {
+        if constexpr (sizeof(T) == 4) return reinterpret_cast<const Quad<T>*>(p)[i];
+        else return {p[i], p[S + i]};
+    }
+    __device__ __forceinline__ void st(int i, const Quad<T>& x) const
+    {
+        if constexpr (sizeof(T) == 4) {
+            reinterpret_cast<Quad<T>*>(p)[i] = x;
+        } else {
+            p[i] = x.a;
+            p[S + i] = x.b;
+        }
+    }
+    __device__ __forceinline__ Pr<T>* end() const { return p + 2 * S; }
+};
+
 // Shared memory of a tile, in quads.
 template <int N, int TX, int TY>
 struct QuadLayout {
@@ -232,6 +255,19 @@ __device__ __forceinline__ Quad<T> quad_flux(const Quad<T>& q, const Phys<T>& ph
     else return qmk(v[2], v[1] * w, fma(v[2], w, p), h);
 }
 
+// Both fluxes of Eq. 4 at one point (q may be f).
+template <class T>
+__device__ __forceinline__ void quad_flux_xy(const Quad<T>& q, const Phys<T>& ph, Quad<T>& f, Quad<T>& g)
+{
+    T v[4];
+    qget(q, v);
+    const T r = rcp_of<true>(v[0]), u = v[1] * r, w = v[2] * r;
+    const T mw = v[1] * w;
+    const T p = (ph.gamma - T(1)) * fma(T(-0.5), fma(v[1], u, v[2] * w), v[3]), h = v[3] + p;
+    f = qmk(v[1], fma(v[1], u, p), mw, h * u);
+    g = qmk(v[2], mw, fma(v[2], w, p), h * w);
+}
+
 // Twice the common flux through a face between the lower state m and the
 // upper state p (the factor 1/2 joins the jump's subtraction, half_jump).
 template <int FLUX, int DIR, class T>
@@ -261,16 +297,16 @@ __device__ __forceinline__ Quad<T> half_jump(const Quad<T>& G2, const Quad<T>& f
 // fluxes flo, fhi that the common fluxes are compared with (joined operator:
 // those of the first and last point; else of the edges) of the line x
 // (consumed).
-template <int N, int DIR, int DIV>
-__device__ __forceinline__ void quad_line(const QuadTab<float>& t, const Phys<float>& ph, Quad<float> (&x)[N], Quad<float> (&r)[N],
-                                          Quad<float>& lo, Quad<float>& hi, Quad<float>& flo, Quad<float>& fhi)
+template <int N, int DIR, int DIV, class T>
+__device__ __forceinline__ void quad_line(const QuadTab<T>& t, const Phys<T>& ph, Quad<T> (&x)[N], Quad<T> (&r)[N],
+                                          Quad<T>& lo, Quad<T>& hi, Quad<T>& flo, Quad<T>& fhi)
 {
     lo = edge_lo<N>(t, x);
     hi = edge_hi<N>(t, x);
     if constexpr (DIV == DIV_LP) {
 #pragma unroll
         for (int a = 0; a < N; ++a) x[a] = quad_flux<DIR>(x[a], ph);
-        if constexpr (quad_joined<float>(N)) {
+        if constexpr (quad_joined<T>(N)) {
             flo = x[0];
             fhi = x[N - 1];
         } else {
@@ -279,11 +315,11 @@ __device__ __forceinline__ void quad_line(const QuadTab<float>& t, const Phys<fl
         }
         line_derivative<N>(t, x, r);
     } else {
-        Quad<float> dq[N];
+        Quad<T> dq[N];
         line_derivative<N>(t, x, dq);
 #pragma unroll
         for (int a = 0; a < N; ++a) {
-            float q[4], d[4], o[4];
+            T q[4], d[4], o[4];
             qget(x[a], q);
             qget(dq[a], d);
             flux_jvp<EQ_EULER, DIR, true>(q, d, ph, o);
