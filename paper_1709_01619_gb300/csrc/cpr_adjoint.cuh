@@ -1,4 +1,5 @@
-// cpr_adjoint.cuh -- transpose of the CPR residual (discrete adjoint).
+// cpr_adjoint.cuh -- transpose of the CPR residual (discrete adjoint): the
+// method, and the kernel of advection (Euler: cpr_adjoint_quad.cuh).
 //
 // qbar = (dR/dq)^T rbar for the LP divergence (Sec. 2.2, Eq. 16-17 with the
 // flux interpolant differentiated), written as a gather: every element
@@ -41,7 +42,7 @@ struct VjpArgs {
     T rhx2, rhy2;
     Phys<T> ph;
     Tab<T> tab;
-    T M[kMaxN][kMaxN];
+    T MT[kMaxN][kMaxN];  // MT[l][a] = M_al
 };
 
 template <int N, int V, int TX, int TY>
@@ -69,10 +70,9 @@ struct VjpLayout {
 };
 
 // Resident CTAs per SM the register budget is sized for (0: no bound): in
-// FP32, for tiles of 32 elements, as many as the shared memory holds
-// (p = 2: 8, p = 3: 6 with 16 bytes of spills, p = 4: 4; unbounded, the
-// registers allowed 7, 5 and 3; 1024^2 p = 3: 0.364 -> 0.351 ms per
-// launch), scaled for other tile sizes; FP64 unbounded.
+// FP32 as many tiles of 32 elements as the shared memory of the four-variable
+// kernel held, scaled for other tile sizes (advection, the only equation left
+// to this kernel, uses 32 to 48 registers); FP64 unbounded.
 template <class T, int P, int ELEMS>
 constexpr int vjp_min_blocks()
 {
@@ -206,9 +206,9 @@ cpr_residual_vjp_kernel(const VjpArgs<T> A)
             T fb[V];
 #pragma unroll
             for (int v = 0; v < V; ++v) {
-                T s = xb[0][v] * A.M[0][l];
+                T s = xb[0][v] * A.MT[l][0];
 #pragma unroll
-                for (int a = 1; a < N; ++a) s = fma(xb[a][v], A.M[a][l], s);
+                for (int a = 1; a < N; ++a) s = fma(xb[a][v], A.MT[l][a], s);
                 fb[v] = s;
                 qrow[l][v] = T(0);
             }
@@ -244,9 +244,9 @@ cpr_residual_vjp_kernel(const VjpArgs<T> A)
             T gb[V], c[V];
 #pragma unroll
             for (int v = 0; v < V; ++v) {
-                T s = xb[0][v] * A.M[0][l];
+                T s = xb[0][v] * A.MT[l][0];
 #pragma unroll
-                for (int b = 1; b < N; ++b) s = fma(xb[b][v], A.M[b][l], s);
+                for (int b = 1; b < N; ++b) s = fma(xb[b][v], A.MT[l][b], s);
                 gb[v] = s;
                 c[v] = T(0);
             }

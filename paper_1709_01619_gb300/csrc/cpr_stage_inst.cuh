@@ -8,7 +8,7 @@
 #include "cpr_launch.h"
 #include "cpr_tabconv.cuh"
 #include "cpr_stage.cuh"
-#include "cpr_adjoint.cuh"
+#include "cpr_adjoint_quad.cuh"
 
 namespace cpr {
 
@@ -217,26 +217,27 @@ cudaError_t prepare_stage_p(const LaunchCfg& c)
     return stage_dispatch<T, P>(c, A, 0, 0, true);
 }
 
-// Tile of the adjoint kernel: FP32 8 x 4 elements (twice as many CTAs per
-// SM as 8 x 8 ones in the same shared memory: 1024^2 p = 3 0.441 -> 0.411 ms
-// per launch; the height is overridable for tuning sweeps); FP64 8 x 8, or
+// Tile of the adjoint kernels: 8 x 4 elements (twice as many CTAs per SM as
+// 8 x 8 ones in the same shared memory: 1024^2 p = 3 FP32 0.441 -> 0.411 ms per
+// launch of the kernel with one word per variable); FP64 advection 8 x 8, or
 // 8 x 4 where 8 x 8 would exceed the shared memory of one CTA.
-#ifndef CPR_VJP_TILE_Y
-#define CPR_VJP_TILE_Y 4
-#endif
-template <class T, int P>
+template <class T, int P, int EQ>
 struct VjpTile {
     static constexpr int X = 8;
-    static constexpr int Y = sizeof(T) == 8 ? (P == 4 ? 4 : 8) : CPR_VJP_TILE_Y;
+    static constexpr int Y = sizeof(T) == 8 && EQ == EQ_ADV && P < 4 ? 8 : 4;
 };
 
 template <class T, int P, int EQ, int FLUX>
 static cudaError_t vjp_one(const LaunchCfg& c, const VjpPtrs& b, cudaStream_t s, bool prep)
 {
     constexpr int N = P + 1, V = NVars<EQ>::value;
-    constexpr int TX = VjpTile<T, P>::X, TY = VjpTile<T, P>::Y;
-    auto kern = cpr_residual_vjp_kernel<T, P, EQ, FLUX, TX, TY>;
-    const size_t smem = sizeof(T) * VjpLayout<N, V, TX, TY>::TOTAL;
+    constexpr int TX = VjpTile<T, P, EQ>::X, TY = VjpTile<T, P, EQ>::Y;
+    auto kern = [] {
+        if constexpr (EQ == EQ_EULER) return cpr_vjp_quad_kernel<T, P, TX, TY>;
+        else return cpr_residual_vjp_kernel<T, P, EQ, FLUX, TX, TY>;
+    }();
+    const size_t smem = EQ == EQ_EULER ? sizeof(Quad<T>) * VjpQuadLayout<T, N, TX, TY>::TOTAL
+                                       : sizeof(T) * VjpLayout<N, V, TX, TY>::TOTAL;
     if (prep) return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     VjpArgs<T> A;
     A.q = static_cast<const T*>(b.q);
@@ -263,9 +264,9 @@ static cudaError_t vjp_one(const LaunchCfg& c, const VjpPtrs& b, cudaStream_t s,
     A.tab = host_tab<T>(c.tab);
     for (int a = 0; a < kMaxN; ++a)
         for (int l = 0; l < kMaxN; ++l)
-            A.M[a][l] = (a < N && l < N)
-                            ? T(c.tab.D[a][l] - c.tab.lm[l] * c.tab.dgl[a] - c.tab.lp[l] * c.tab.dgr[a])
-                            : T(0);
+            A.MT[l][a] = (a < N && l < N)
+                             ? T(c.tab.D[a][l] - c.tab.lm[l] * c.tab.dgl[a] - c.tab.lp[l] * c.tab.dgr[a])
+                             : T(0);
     const int ctas = A.tiles_x * ((c.ny + TY - 1) / TY);
     kern<<<ctas, TX * TY * N, smem, s>>>(A);
     return cudaGetLastError();

@@ -195,15 +195,15 @@ struct QuadLayout {
 
 // Row of N values of every variable (point offset off) as quads; addb adds
 // the increment array.
-template <int N>
-__device__ __forceinline__ void load_row_quads(const float* __restrict__ q, const float* __restrict__ qb, bool addb,
-                                               long long npts, long long off, Quad<float> (&x)[N])
+template <int N, class T>
+__device__ __forceinline__ void load_row_quads(const T* __restrict__ q, const T* __restrict__ qb, bool addb,
+                                               long long npts, long long off, Quad<T> (&x)[N])
 {
-    float r[4][N];
+    T r[4][N];
 #pragma unroll
     for (int v = 0; v < 4; ++v) gload_row<N>(q + v * npts + off, r[v]);
     if (addb) {
-        float b[4][N];
+        T b[4][N];
 #pragma unroll
         for (int v = 0; v < 4; ++v) gload_row<N>(qb + v * npts + off, b[v]);
 #pragma unroll
@@ -216,17 +216,17 @@ __device__ __forceinline__ void load_row_quads(const float* __restrict__ q, cons
 }
 
 // Column of N values (stride N) of every variable as quads.
-template <int N>
-__device__ __forceinline__ void load_col_quads(const float* __restrict__ q, const float* __restrict__ qb, bool addb,
-                                               long long npts, long long off, Quad<float> (&x)[N])
+template <int N, class T>
+__device__ __forceinline__ void load_col_quads(const T* __restrict__ q, const T* __restrict__ qb, bool addb,
+                                               long long npts, long long off, Quad<T> (&x)[N])
 {
-    float r[4][N];
+    T r[4][N];
 #pragma unroll
     for (int v = 0; v < 4; ++v)
 #pragma unroll
         for (int l = 0; l < N; ++l) r[v][l] = q[v * npts + off + l * N];
     if (addb) {
-        float b[4][N];
+        T b[4][N];
 #pragma unroll
         for (int v = 0; v < 4; ++v)
 #pragma unroll

@@ -1,4 +1,4 @@
-"""The tiles of the FP64 Euler kernel at their edges:
+"""The tiles of the FP64 Euler and the adjoint kernels at their edges:
 grids smaller than a tile, equal to one, one element more, and large enough
 for the FP64 rule to pick each of its tiles (4 x 2 for p = 4, 4 x 4, 8 x 4),
 with both kinds of boundary, against the FP64 oracle.
@@ -40,3 +40,19 @@ def test_euler_fp64(p, div, flux):
     for k, size in enumerate(SMALL + [(21, 19), (48, 40)]):
         check(nat.F64, p, size, BC[k % 4], eqn=nat.EULER, pts=k % 2, div=div, flux=flux)
     check(nat.F64, p, LARGE[p], (0, 1), eqn=nat.EULER, div=div, flux=flux)
+
+
+@pytest.mark.parametrize("p", [1, 2, 3, 4])
+@pytest.mark.parametrize("dtype", [nat.F64, nat.F32])
+def test_euler_adjoint(p, dtype):
+    for k, size in enumerate(SMALL + [(21, 18)]):
+        bc = BC[k % 4]
+        c, o = make(dtype, eqn=nat.EULER, nx=size[0], ny=size[1], p=p, x1=6.0, y1=5.0, bc_x=bc[0], bc_y=bc[1],
+                    pts=k % 2)
+        q = rough_state(o, 9)
+        w = np.random.default_rng(k).standard_normal(q.shape)
+        if dtype == nat.F32:
+            q, w = q.astype(np.float32).astype(np.float64), w.astype(np.float32).astype(np.float64)
+        with nat.Context(c) as ctx:
+            got = host(ctx.residual_vjp(to_dev(q, c), to_dev(w, c)))
+        assert rel_l2(got, oracle.residual_vjp(o, q, w)) <= (TOL64 if dtype == nat.F64 else TOL32)
