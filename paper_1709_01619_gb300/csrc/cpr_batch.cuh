@@ -105,7 +105,9 @@ __device__ __forceinline__ void batch_item(const BatchArgs<T>& B, int w, StageAr
         s_n = I.ntiles;
     }
     __syncthreads();
-    if constexpr (sizeof(T) == 8 && EQ == EQ_EULER)
+    if constexpr (EQ == EQ_ADV)
+        stage_tile_adv<T, P, TX, TY>(sA, B.tab, B.qx, s_t, threadIdx.x, smem_raw, s_n);
+    else if constexpr (sizeof(T) == 8)
         stage_tile_f64<P, DIV, FLUX, TX, TY>(sA, B.tab, B.qx, s_t, threadIdx.x, smem_raw, s_n);
     else if constexpr (stage_quad<T, EQ, DELTA>)
         stage_tile_quad<P, DIV, FLUX, TX, TY, false, 0>(sA, B.tab, B.qx, s_t, threadIdx.x, smem_raw, s_n);

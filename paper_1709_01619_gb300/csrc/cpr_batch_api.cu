@@ -142,7 +142,7 @@ cudaError_t batch_launch(cpr_batch* b, Group& g, int fam, int grid, int mode, in
     B.swap = swap;
     B.tab = cpr::host_tab<T>(b->lcs[g.members[0]].tab);
     B.tp = cpr::host_tabpr<T>(b->lcs[g.members[0]].tab);
-    B.qx.tab = cpr::host_quadtab<T>(b->lcs[g.members[0]].tab, cpr::quad_joined<T>(g.p + 1));
+    B.qx.tab = cpr::host_quadtab<T>(b->lcs[g.members[0]].tab, b->V == 1 || cpr::quad_joined<T>(g.p + 1));
     const LaunchCfg& lc = b->lcs[g.members[0]];
     return fam == 0 ? cpr::batch_fam<T, 0>(g.p, lc.eqn, lc.flux, B, grid, s, 0, nullptr)
                     : cpr::batch_fam<T, 1>(g.p, lc.eqn, lc.flux, B, grid, s, 0, nullptr);

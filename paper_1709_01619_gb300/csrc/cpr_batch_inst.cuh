@@ -28,11 +28,10 @@ static cudaError_t batch_one(const BatchArgs<T>& B, int grid, cudaStream_t s, in
 }
 
 template <class T, int P, int FAM>
-static cudaError_t batch_p(int eqn, int flux, const BatchArgs<T>& B, int grid, cudaStream_t s, int what, int* occ)
+static cudaError_t batch_p(int eqn, const BatchArgs<T>& B, int grid, cudaStream_t s, int what, int* occ)
 {
     if (eqn == EQ_EULER) return batch_one<T, P, EQ_EULER, FLUX_RUSANOV, FAM>(B, grid, s, what, occ);
-    if (flux == FLUX_UPWIND) return batch_one<T, P, EQ_ADV, FLUX_UPWIND, FAM>(B, grid, s, what, occ);
-    return batch_one<T, P, EQ_ADV, FLUX_RUSANOV, FAM>(B, grid, s, what, occ);
+    return batch_one<T, P, EQ_ADV, FLUX_UPWIND, FAM>(B, grid, s, what, occ);  // Rusanov is the same flux
 }
 
 template <class T, int FAM>
@@ -40,10 +39,10 @@ cudaError_t batch_fam(int p, int eqn, int flux, const BatchArgs<T>& B, int grid,
                       int* occ)
 {
     switch (p) {
-    case 1: return batch_p<T, 1, FAM>(eqn, flux, B, grid, s, what, occ);
-    case 2: return batch_p<T, 2, FAM>(eqn, flux, B, grid, s, what, occ);
-    case 3: return batch_p<T, 3, FAM>(eqn, flux, B, grid, s, what, occ);
-    case 4: return batch_p<T, 4, FAM>(eqn, flux, B, grid, s, what, occ);
+    case 1: return batch_p<T, 1, FAM>(eqn, B, grid, s, what, occ);
+    case 2: return batch_p<T, 2, FAM>(eqn, B, grid, s, what, occ);
+    case 3: return batch_p<T, 3, FAM>(eqn, B, grid, s, what, occ);
+    case 4: return batch_p<T, 4, FAM>(eqn, B, grid, s, what, occ);
     default: return cudaErrorInvalidValue;
     }
 }

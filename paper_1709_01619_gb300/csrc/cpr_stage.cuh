@@ -362,6 +362,7 @@ constexpr int stage_threads(int n) { return (n + 31) / 32 * 32; }
 
 }  // namespace cpr
 
+#include "cpr_stage_adv.cuh"
 #include "cpr_stage_f64.cuh"
 #include "cpr_stage_quad.cuh"
 
@@ -376,7 +377,8 @@ constexpr bool stage_quad = sizeof(T) == 4 && EQ == EQ_EULER && !DELTA;
 template <class T, int P, int EQ, int TX, int TY, bool DELTA>
 constexpr size_t stage_smem()
 {
-    if constexpr (sizeof(T) == 8 && EQ == EQ_EULER) return sizeof(Quad<double>) * F64Layout<P + 1, TX, TY>::TOTAL;
+    if constexpr (EQ == EQ_ADV) return sizeof(T) * AdvLayout<P + 1, TX, TY>::TOTAL;
+    else if constexpr (sizeof(T) == 8) return sizeof(Quad<double>) * F64Layout<P + 1, TX, TY>::TOTAL;
     else if constexpr (stage_quad<T, EQ, DELTA>) return sizeof(Quad<float>) * QuadLayout<P + 1, TX, TY>::TOTAL;
     else return sizeof(T) * StageLayout<P + 1, NVars<EQ>::value, TX, TY, DELTA>::TOTAL;
 }

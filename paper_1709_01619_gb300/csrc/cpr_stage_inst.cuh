@@ -48,19 +48,22 @@ static cudaError_t with_quad_kernel(int mode, bool wide, bool shared, F&& f)
 }
 
 // The tile of a single FP64 problem.  A stage takes the time of the scheduler
-// with most warps (cpr_stage_f64.cuh): of the tiles, the one with the fewest
-// warps on the busiest scheduler, each step down counted 10 % dearer for its
-// longer boundary.  An instance of a batch (sms 0) takes the largest.
+// with most warps (cpr_stage_f64.cuh): of n tiles (size(k, tx, ty) gives their
+// elements and returns their warps), the one with the fewest warps on the
+// busiest scheduler, each step down counted 10 % dearer for its longer
+// boundary.  An instance of a batch (sms 0) takes the largest.
 // us per Euler stage, p = 3: 16^2 elements 16.7 (4 x 4), 64^2 26.4, 96^2 45.9
 // (8 x 8 tiles, one thread for a row and a column: 36 at every size below 64^2).
-inline int f64_tile(const LaunchCfg& c)
+template <class F>
+inline int f64_tile(const LaunchCfg& c, int n, F&& size)
 {
     int best = 0;
     double cost = 0.0, dearer = 1.0;
-    for (int k = 0; c.sms > 0 && k < f64_tiles(c.p); ++k, dearer *= 1.1) {
-        const int tx = f64_tile_x(k), ty = f64_tile_y(k);
+    for (int k = 0; c.sms > 0 && k < n; ++k, dearer *= 1.1) {
+        int tx, ty;
+        const int tile_warps = size(k, &tx, &ty);
         const long long ctas = (long long)((c.nx + tx - 1) / tx) * ((c.ny + ty - 1) / ty);
-        const long long warps = (ctas + c.sms - 1) / c.sms * (2 * f64_role_threads(c.p, tx, ty) / 32);
+        const long long warps = (ctas + c.sms - 1) / c.sms * tile_warps;
         const double w = (double)((warps + 3) / 4) * dearer;
         if (k == 0 || w < cost) {
             best = k;
@@ -86,16 +89,48 @@ static cudaError_t stage_f64_tile(const LaunchCfg& c, StageArgs<double> A, cudaS
 template <int P, int DIV, int FLUX>
 static cudaError_t stage_f64(const LaunchCfg& c, const StageArgs<double>& A, cudaStream_t s, bool prep)
 {
-    const int k = f64_tile(c);
+    const int k = f64_tile(c, f64_tiles(P), [](int i, int* tx, int* ty) {
+        *tx = f64_tile_x(i);
+        *ty = f64_tile_y(i);
+        return 2 * f64_role_threads(P, *tx, *ty) / 32;
+    });
     if constexpr (f64_tiles(P) > 2)
         if (k == 2) return stage_f64_tile<P, DIV, FLUX, 2>(c, A, s, prep);
     return k == 1 ? stage_f64_tile<P, DIV, FLUX, 1>(c, A, s, prep) : stage_f64_tile<P, DIV, FLUX, 0>(c, A, s, prep);
 }
 
+template <class T, int P, int K>
+static cudaError_t stage_adv_tile(const LaunchCfg& c, StageArgs<T> A, cudaStream_t s, bool prep)
+{
+    constexpr int TX = adv_tile_x(P, K), TY = adv_tile_y(P, K);
+    const size_t smem = stage_smem<T, P, EQ_ADV, TX, TY, false>();
+    auto kern = cpr_stage_adv_kernel<T, P, TX, TY>;
+    if (prep) return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    A.tiles_x = (c.nx + TX - 1) / TX;
+    div_magic((unsigned)A.tiles_x, &A.qx.tx_magic, &A.qx.tx_shift);
+    kern<<<A.tiles_x * ((c.ny + TY - 1) / TY), stage_threads(TX * TY * (P + 1)), smem, s>>>(A);
+    return cudaGetLastError();
+}
+
+template <class T, int P>
+static cudaError_t stage_adv(const LaunchCfg& c, const StageArgs<T>& A, cudaStream_t s, bool prep)
+{
+    if constexpr (sizeof(T) == 8) {
+        const int k = f64_tile(c, 2, [](int i, int* tx, int* ty) {
+            *tx = adv_tile_x(P, i);
+            *ty = adv_tile_y(P, i);
+            return stage_threads(*tx * *ty * (P + 1)) / 32;
+        });
+        if (k == 1) return stage_adv_tile<T, P, 1>(c, A, s, prep);
+    }
+    return stage_adv_tile<T, P, 0>(c, A, s, prep);
+}
+
 template <class T, int P, int EQ, int DIV, int FLUX>
 static cudaError_t stage_one(const LaunchCfg& c, const StageArgs<T>& A, int ctas, cudaStream_t s, bool prep)
 {
-    if constexpr (sizeof(T) == 8 && EQ == EQ_EULER) return stage_f64<P, DIV, FLUX>(c, A, s, prep);
+    if constexpr (EQ == EQ_ADV) return stage_adv<T, P>(c, A, s, prep);
+    else if constexpr (sizeof(T) == 8) return stage_f64<P, DIV, FLUX>(c, A, s, prep);
     else {
     constexpr int N = P + 1, V = NVars<EQ>::value;
     constexpr int TX = stage_tile_x(P), TY = stage_tile_y(P);
@@ -153,13 +188,8 @@ static cudaError_t stage_one(const LaunchCfg& c, const StageArgs<T>& A, int ctas
 template <class T, int P>
 static cudaError_t stage_dispatch(const LaunchCfg& c, const StageArgs<T>& A, int ctas, cudaStream_t s, bool prep)
 {
-    if (c.eqn == EQ_ADV) {
-        if (c.flux == FLUX_UPWIND)
-            return c.div == DIV_LP ? stage_one<T, P, EQ_ADV, DIV_LP, FLUX_UPWIND>(c, A, ctas, s, prep)
-                                   : stage_one<T, P, EQ_ADV, DIV_CHAIN, FLUX_UPWIND>(c, A, ctas, s, prep);
-        return c.div == DIV_LP ? stage_one<T, P, EQ_ADV, DIV_LP, FLUX_RUSANOV>(c, A, ctas, s, prep)
-                               : stage_one<T, P, EQ_ADV, DIV_CHAIN, FLUX_RUSANOV>(c, A, ctas, s, prep);
-    }
+    // advection: every divergence and flux is one operator (cpr_stage_adv.cuh)
+    if (c.eqn == EQ_ADV) return stage_one<T, P, EQ_ADV, DIV_LP, FLUX_UPWIND>(c, A, ctas, s, prep);
     if (c.flux == FLUX_ROE)
         return c.div == DIV_LP ? stage_one<T, P, EQ_EULER, DIV_LP, FLUX_ROE>(c, A, ctas, s, prep)
                                : stage_one<T, P, EQ_EULER, DIV_CHAIN, FLUX_ROE>(c, A, ctas, s, prep);
@@ -197,7 +227,7 @@ static StageArgs<T> make_stage_args(const LaunchCfg& c, int mode, const StagePtr
     A.ph.ay = T(c.ay);
     A.tab = host_tab<T>(c.tab);
     A.tp = host_tabpr<T>(c.tab);
-    A.qx.tab = host_quadtab<T>(c.tab, c.div == DIV_LP && quad_joined<T>(c.p + 1));
+    A.qx.tab = host_quadtab<T>(c.tab, c.eqn == EQ_ADV || (c.div == DIV_LP && quad_joined<T>(c.p + 1)));
     div_magic((unsigned)A.tiles_x, &A.qx.tx_magic, &A.qx.tx_shift);
     return A;
 }

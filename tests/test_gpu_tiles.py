@@ -1,4 +1,4 @@
-"""The tiles of the FP64 Euler and the adjoint kernels at their edges:
+"""The tiles of the FP64 Euler, advection and adjoint kernels at their edges:
 grids smaller than a tile, equal to one, one element more, and large enough
 for the FP64 rule to pick each of its tiles (4 x 2 for p = 4, 4 x 4, 8 x 4),
 with both kinds of boundary, against the FP64 oracle.
@@ -40,6 +40,15 @@ def test_euler_fp64(p, div, flux):
     for k, size in enumerate(SMALL + [(21, 19), (48, 40)]):
         check(nat.F64, p, size, BC[k % 4], eqn=nat.EULER, pts=k % 2, div=div, flux=flux)
     check(nat.F64, p, LARGE[p], (0, 1), eqn=nat.EULER, div=div, flux=flux)
+
+
+@pytest.mark.parametrize("p", [1, 2, 3, 4])
+@pytest.mark.parametrize("dtype", [nat.F64, nat.F32])
+@pytest.mark.parametrize("velocity", [(0.7, 1.3), (-0.7, 0.4), (0.6, -1.1), (-0.3, -0.9), (0.0, 0.5)])
+def test_advection(p, dtype, velocity):
+    for k, size in enumerate(SMALL + [(21, 19), LARGE[p]]):
+        check(dtype, p, size, BC[k % 4], eqn=nat.ADVECTION, pts=k % 2, div=k // 2 % 2,
+              flux=(nat.UPWIND, nat.RUSANOV)[k % 2], ax=velocity[0], ay=velocity[1])
 
 
 @pytest.mark.parametrize("p", [1, 2, 3, 4])
