@@ -147,6 +147,7 @@ __global__ void __launch_bounds__(TX * TY * (P + 1), vjp_quad_min_blocks<T>(P)) 
     const QuadArr<T, L::YH> yHq{yTw.end()}, yHw{yHq.end()};
     const QuadArr<T, L::EF> xQ{yHw.end()}, yQ{xQ.end()}, yB{yQ.end()};  // right, top, bottom face
 
+    grid_order();
     const int tid = threadIdx.x;
     const int tj = blockIdx.x / A.tiles_x;
     const int i0 = (blockIdx.x - tj * A.tiles_x) * TX, j0 = tj * TY;

@@ -525,6 +525,15 @@ extern "C" cpr_status cpr_get_time(cpr_ctx* c, double* t, long long* steps)
     return CPR_OK;
 }
 
+// Launches behind another kernel of this call on the context's stream: from
+// its construction to the end of its scope.  Not the first launch of a call,
+// whose predecessor is the caller's.
+struct Behind {
+    LaunchCfg& lc;
+    explicit Behind(cpr_ctx* c) : lc(c->lc) { lc.behind = true; }
+    ~Behind() { lc.behind = false; }
+};
+
 static cudaError_t vjp(cpr_ctx* c, const cpr::VjpPtrs& b, cudaStream_t s)
 {
     return c->cfg.dtype == CPR_F32 ? cpr::launch_vjp<float>(c->lc, b, s, false)
@@ -577,6 +586,7 @@ static cpr_status step_vjp_chain(cpr_ctx* c, const void* q, const void* q1, cons
     if (!c->adj2) CPR_CUDA(c, cudaMalloc(&c->adj2, bytes));
     cpr::VjpPtrs b2{q2, qbar_out, c->adj1, qbar_out, nullptr, nullptr, 2.0 / 3.0, 0.0, 0.0, 2.0 / 3.0 * dt};
     CPR_CUDA(c, vjp(c, b2, c->stream));
+    Behind behind(c);
     cpr::VjpPtrs b1{q1, c->adj1, c->adj2, c->adj1, nullptr, nullptr, 0.25, 0.0, 0.0, 0.25 * dt};
     CPR_CUDA(c, vjp(c, b1, c->stream));
     cpr::VjpPtrs b0{q, c->adj2, qbar_in, qbar_out, c->adj1, c->adj2, 1.0 / 3.0, 0.75, 1.0, dt};
@@ -590,6 +600,7 @@ static cpr_status so_stages(cpr_ctx* c, const void* q, void* q1, void* q2, void*
     ctrl_configure_kernel<<<1, 1, 0, c->stream>>>(c->ctrl, dt, 0.0, 0.0);
     CPR_CUDA(c, cudaGetLastError());
     CPR_CUDA(c, stage(c, cpr::MODE_SO1, q, nullptr, q1, nullptr, false, c->stream));
+    Behind behind(c);
     CPR_CUDA(c, stage(c, cpr::MODE_SO2, q1, q, q2, nullptr, false, c->stream));
     if (q_next) CPR_CUDA(c, stage(c, cpr::MODE_SO3, q2, q, q_next, nullptr, false, c->stream));
     return CPR_OK;

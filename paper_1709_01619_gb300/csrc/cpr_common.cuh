@@ -68,6 +68,25 @@ struct Ctrl {
                               // non-negative double); 0 between kernels
 };
 
+// Programmatic dependent launch.  A kernel launched behind another one of its
+// stream (LaunchCfg::behind) may start while that one still runs: its CTAs
+// take the slots that the last CTAs of the other leave free, and wait here
+// until the other has finished and its writes are visible.  Every CTA of such
+// a kernel calls this before its first access to global memory, so that the
+// order of the accesses is that of ordinary launches; then it lets the next
+// kernel of the stream start the same way.  Launched without the attribute,
+// both instructions do nothing.
+//
+// The kernels that the step adjoint of the Euler equations launches one by one
+// gain from it (gradient through 20 steps, 256^2 p = 3: 2.97 -> 2.85 ms); those
+// of the step graphs do not (128^2 p = 3 FP64 3.09 -> 3.11 ms, FV 1536^2 1.334 ->
+// 1.353; 128^2 FP32 1.103 -> 1.119 with the two instructions alone).
+__device__ __forceinline__ void grid_order()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
+}
+
 // Physics in the arithmetic type T.
 template <class T>
 struct Phys {

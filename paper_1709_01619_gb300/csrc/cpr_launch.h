@@ -30,6 +30,8 @@ struct LaunchCfg {
     int sms;                // SMs of the device: a stage launch of at most two CTAs per SM takes
                             // the instantiation compiled for two resident CTAs (0: never)
     bool shared;            // an instance of a batch: its launches share the SMs with other instances
+    bool behind;            // the launch follows another kernel of this library on its stream: it may
+                            // start while that one drains (grid_order)
     int nx, ny, bcx, bcy;
     long long ne, npts;
     double hx, hy, gamma, ax, ay, tvb_M, lim_eps;
@@ -38,6 +40,24 @@ struct LaunchCfg {
     int* marks;        // limiter marks
     double* partials;  // norms partials
 };
+
+// Launch of a kernel that begins with grid_order().
+template <class... K, class... A>
+cudaError_t launch_ordered(const LaunchCfg& c, void (*k)(K...), int grid, int block, size_t smem, cudaStream_t s,
+                           const A&... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = c.behind ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k, args...);
+}
 
 // SM count of the current device (0 when it cannot be queried).
 inline int current_sm_count()

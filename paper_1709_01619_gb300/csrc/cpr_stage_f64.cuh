@@ -8,8 +8,9 @@
 //   - the operations are few: the pressure, velocities and 1 / rho of a point
 //     serve the fluxes of both directions (LP divergence), the line operators
 //     take the mirrored, joined form (line_derivative), reciprocals and square
-//     roots are the short ones of cpr_common.cuh: 130 per point for p = 3
-//     instead of about 275;
+//     roots are the short ones of cpr_common.cuh: 140 operations or 222 flops
+//     per point and stage for p = 3, counted, against the general tile's 297
+//     flops;
 //   - the warps are many and alike: the threads of a CTA have one of two roles,
 //     x-lines (rows) and y-lines (columns), and share the points of a row in
 //     the phases that work on points, so that a thread has half the
@@ -317,6 +318,7 @@ template <int P, int DIV, int FLUX, int TX, int TY, int MINB>
 __global__ void __launch_bounds__(2 * f64_role_threads(P, TX, TY), MINB) cpr_stage_f64_kernel(const StageArgs<double> A)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    grid_order();
     stage_tile_f64<P, DIV, FLUX, TX, TY>(A, A.tab, A.qx, blockIdx.x, threadIdx.x, smem_raw, gridDim.x);
 }
 

@@ -82,8 +82,7 @@ static cudaError_t stage_f64_tile(const LaunchCfg& c, StageArgs<double> A, cudaS
     if (prep) return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     A.tiles_x = (c.nx + TX - 1) / TX;
     div_magic((unsigned)A.tiles_x, &A.qx.tx_magic, &A.qx.tx_shift);
-    kern<<<A.tiles_x * ((c.ny + TY - 1) / TY), 2 * f64_role_threads(P, TX, TY), smem, s>>>(A);
-    return cudaGetLastError();
+    return launch_ordered(c, kern, A.tiles_x * ((c.ny + TY - 1) / TY), 2 * f64_role_threads(P, TX, TY), smem, s, A);
 }
 
 template <int P, int DIV, int FLUX>
@@ -172,6 +171,9 @@ static cudaError_t stage_one(const LaunchCfg& c, const StageArgs<T>& A, int ctas
     if constexpr (QUAD) {
         if (A.mode != MODE_RESIDUAL) {
             auto launch = [&](auto k) {
+                // a kernel compiled for its Shu-Osher stage: in order behind another
+                if (DIV == DIV_LP && FLUX == FLUX_RUSANOV && !c.shared && quad_ordered(A.mode))
+                    return launch_ordered(c, k, ctas, NT, smem_q, s, A);
                 k<<<ctas, NT, smem_q, s>>>(A);
                 return cudaGetLastError();
             };
@@ -298,6 +300,7 @@ static cudaError_t vjp_one(const LaunchCfg& c, const VjpPtrs& b, cudaStream_t s,
                              ? T(c.tab.D[a][l] - c.tab.lm[l] * c.tab.dgl[a] - c.tab.lp[l] * c.tab.dgr[a])
                              : T(0);
     const int ctas = A.tiles_x * ((c.ny + TY - 1) / TY);
+    if constexpr (EQ == EQ_EULER) return launch_ordered(c, kern, ctas, TX * TY * N, smem, s, A);
     kern<<<ctas, TX * TY * N, smem, s>>>(A);
     return cudaGetLastError();
 }

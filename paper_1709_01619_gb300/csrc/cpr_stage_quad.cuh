@@ -620,11 +620,16 @@ constexpr int quad_min_blocks()
     return P == 4 && !WIDE ? 128 / ELEMS : stage_min_blocks<float, P + 1, WIDE, ELEMS>();
 }
 
+// The kernels that the step adjoint launches behind one another: those compiled
+// for a Shu-Osher stage.
+__host__ __device__ constexpr bool quad_ordered(int mode) { return mode >= MODE_SO1 && mode <= MODE_SO3; }
+
 template <int P, int DIV, int FLUX, int TX, int TY, int MINB, int MODE>
 __global__ void __launch_bounds__(TX * TY * (P + 1), MINB) cpr_stage_quad_kernel(const StageArgs<float> A)
 {
     static_assert((TX * TY * (P + 1)) % 32 == 0, "whole warps: the warp-level reductions use every lane");
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    if constexpr (quad_ordered(MODE)) grid_order();
     stage_tile_quad<P, DIV, FLUX, TX, TY, false, MODE>(A, A.tab, A.qx, blockIdx.x, threadIdx.x, smem_raw, gridDim.x);
 }
 
