@@ -218,7 +218,7 @@ cpr_fv_stage_kernel(const StageArgs<T> A, const int rows)
         if (mode == MODE_SO2 || mode == MODE_INC2) w *= T(0.25);
         if (mode == MODE_SO3 || mode == MODE_INC3) w *= T(2.0 / 3.0);
         // one half of 1 / dx, 1 / dy: the fluxes are doubled
-        const T sx = T(-0.25) * A.rhx2 * w, sy = T(-0.25) * A.rhy2 * w;
+        const T sx = T(-0.25) * A.rhx2, sy = T(-0.25) * A.rhy2;
         // row j0 - 1 is there for its upper face only (the same instructions
         // for every face, so that both warps of a face see the same bits)
         for (int j = j0 - 1; j < jend; ++j) {
@@ -242,7 +242,9 @@ cpr_fv_stage_kernel(const StageArgs<T> A, const int rows)
             fv_states<ORDER>(c, dx, fv_down_lane(dx), up, dn);
             const El Fl = fv_face2<EQ, FLUX, 0>(fv_up_lane(up), dn, A.ph);
             El o = fv_scale(sx, fv_diff(fv_down_lane(Fl), Fl));
-            o = fv_axpy(sy, fv_diff(Ghi, Glo), o);
+            // (the step's factor last: rounded into sx and sy it would be an
+            // error common to every element and step, which does not average out)
+            o = fv_scale(w, fv_axpy(sy, fv_diff(Ghi, Glo), o));
             if (mode == MODE_SO1) {
                 o = fv_axpy(T(1), s0, o);
             } else if (mode == MODE_SO2 || mode == MODE_SO3) {
