@@ -321,7 +321,8 @@ constexpr bool stage_delta()
 }
 
 // Resident CTAs per SM the register budget is sized for (FP32: as many as the
-// shared memory allows; FP64: one, two for p = 3).
+// shared memory allows; FP64, in the grouped batch kernels: as the registers
+// allow).
 #ifndef CPR_STAGE_MINB_FP32
 #define CPR_STAGE_MINB_FP32 4
 #endif
