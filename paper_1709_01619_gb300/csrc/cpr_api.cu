@@ -111,11 +111,15 @@ static cudaError_t stage_inc(cpr_ctx* c, int mode, const void* qs, const void* q
     cpr::StagePtrs b{qs, qb, nullptr, out, c->lo, nullptr};
     return cpr::launch_stage<float>(c->lc, mode, b, wave, s);
 }
+// behind: another kernel of the same call precedes this one on the stream (not
+// for the first launch of a call, whose predecessor is the caller's).
 static cudaError_t stage(cpr_ctx* c, int mode, const void* qs, const void* qn, void* out, void* avg, bool wave,
-                         cudaStream_t s)
+                         cudaStream_t s, bool behind = false)
 {
-    return c->cfg.dtype == CPR_F32 ? cpr::launch_stage<float>(c->lc, mode, qs, qn, out, avg, wave, s)
-                                   : cpr::launch_stage<double>(c->lc, mode, qs, qn, out, avg, wave, s);
+    LaunchCfg lc = c->lc;
+    lc.behind = behind;
+    return c->cfg.dtype == CPR_F32 ? cpr::launch_stage<float>(lc, mode, qs, qn, out, avg, wave, s)
+                                   : cpr::launch_stage<double>(lc, mode, qs, qn, out, avg, wave, s);
 }
 static cudaError_t averages(cpr_ctx* c, const void* q, void* avg, cudaStream_t s)
 {
@@ -525,19 +529,12 @@ extern "C" cpr_status cpr_get_time(cpr_ctx* c, double* t, long long* steps)
     return CPR_OK;
 }
 
-// Launches behind another kernel of this call on the context's stream: from
-// its construction to the end of its scope.  Not the first launch of a call,
-// whose predecessor is the caller's.
-struct Behind {
-    LaunchCfg& lc;
-    explicit Behind(cpr_ctx* c) : lc(c->lc) { lc.behind = true; }
-    ~Behind() { lc.behind = false; }
-};
-
-static cudaError_t vjp(cpr_ctx* c, const cpr::VjpPtrs& b, cudaStream_t s)
+static cudaError_t vjp(cpr_ctx* c, const cpr::VjpPtrs& b, cudaStream_t s, bool behind = false)
 {
-    return c->cfg.dtype == CPR_F32 ? cpr::launch_vjp<float>(c->lc, b, s, false)
-                                   : cpr::launch_vjp<double>(c->lc, b, s, false);
+    LaunchCfg lc = c->lc;
+    lc.behind = behind;
+    return c->cfg.dtype == CPR_F32 ? cpr::launch_vjp<float>(lc, b, s, false)
+                                   : cpr::launch_vjp<double>(lc, b, s, false);
 }
 
 static cpr_status vjp_check(cpr_ctx* c)
@@ -586,11 +583,10 @@ static cpr_status step_vjp_chain(cpr_ctx* c, const void* q, const void* q1, cons
     if (!c->adj2) CPR_CUDA(c, cudaMalloc(&c->adj2, bytes));
     cpr::VjpPtrs b2{q2, qbar_out, c->adj1, qbar_out, nullptr, nullptr, 2.0 / 3.0, 0.0, 0.0, 2.0 / 3.0 * dt};
     CPR_CUDA(c, vjp(c, b2, c->stream));
-    Behind behind(c);
     cpr::VjpPtrs b1{q1, c->adj1, c->adj2, c->adj1, nullptr, nullptr, 0.25, 0.0, 0.0, 0.25 * dt};
-    CPR_CUDA(c, vjp(c, b1, c->stream));
+    CPR_CUDA(c, vjp(c, b1, c->stream, true));
     cpr::VjpPtrs b0{q, c->adj2, qbar_in, qbar_out, c->adj1, c->adj2, 1.0 / 3.0, 0.75, 1.0, dt};
-    CPR_CUDA(c, vjp(c, b0, c->stream));
+    CPR_CUDA(c, vjp(c, b0, c->stream, true));
     return CPR_OK;
 }
 
@@ -600,9 +596,8 @@ static cpr_status so_stages(cpr_ctx* c, const void* q, void* q1, void* q2, void*
     ctrl_configure_kernel<<<1, 1, 0, c->stream>>>(c->ctrl, dt, 0.0, 0.0);
     CPR_CUDA(c, cudaGetLastError());
     CPR_CUDA(c, stage(c, cpr::MODE_SO1, q, nullptr, q1, nullptr, false, c->stream));
-    Behind behind(c);
-    CPR_CUDA(c, stage(c, cpr::MODE_SO2, q1, q, q2, nullptr, false, c->stream));
-    if (q_next) CPR_CUDA(c, stage(c, cpr::MODE_SO3, q2, q, q_next, nullptr, false, c->stream));
+    CPR_CUDA(c, stage(c, cpr::MODE_SO2, q1, q, q2, nullptr, false, c->stream, true));
+    if (q_next) CPR_CUDA(c, stage(c, cpr::MODE_SO3, q2, q, q_next, nullptr, false, c->stream, true));
     return CPR_OK;
 }
 
