@@ -59,6 +59,16 @@ cudaError_t launch_ordered(const LaunchCfg& c, void (*k)(K...), int grid, int bl
     return cudaLaunchKernelEx(&cfg, k, args...);
 }
 
+// Lets kernel k take `bytes` of dynamic shared memory: nothing to do for what
+// every kernel may have (48 KB with its static part), so that a context does
+// not load kernels which it may never launch.
+template <class K>
+inline cudaError_t allow_smem(K k, size_t bytes)
+{
+    if (bytes <= 46 * 1024) return cudaSuccess;
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
 // SM count of the current device (0 when it cannot be queried).
 inline int current_sm_count()
 {

@@ -79,7 +79,7 @@ static cudaError_t stage_f64_tile(const LaunchCfg& c, StageArgs<double> A, cudaS
     constexpr int TX = f64_tile_x(K), TY = f64_tile_y(K);
     const size_t smem = stage_smem<double, P, EQ_EULER, TX, TY, false>();
     auto kern = cpr_stage_f64_kernel<P, DIV, FLUX, TX, TY, f64_min_blocks(P, K)>;
-    if (prep) return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (prep) return allow_smem(kern, smem);
     A.tiles_x = (c.nx + TX - 1) / TX;
     div_magic((unsigned)A.tiles_x, &A.qx.tx_magic, &A.qx.tx_shift);
     return launch_ordered(c, kern, A.tiles_x * ((c.ny + TY - 1) / TY), 2 * f64_role_threads(P, TX, TY), smem, s, A);
@@ -104,7 +104,7 @@ static cudaError_t stage_adv_tile(const LaunchCfg& c, StageArgs<T> A, cudaStream
     constexpr int TX = adv_tile_x(P, K), TY = adv_tile_y(P, K);
     const size_t smem = stage_smem<T, P, EQ_ADV, TX, TY, false>();
     auto kern = cpr_stage_adv_kernel<T, P, TX, TY>;
-    if (prep) return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (prep) return allow_smem(kern, smem);
     A.tiles_x = (c.nx + TX - 1) / TX;
     div_magic((unsigned)A.tiles_x, &A.qx.tx_magic, &A.qx.tx_shift);
     kern<<<A.tiles_x * ((c.ny + TY - 1) / TY), stage_threads(TX * TY * (P + 1)), smem, s>>>(A);
@@ -154,9 +154,7 @@ static cudaError_t stage_one(const LaunchCfg& c, const StageArgs<T>& A, int ctas
     constexpr int WIDE_PER_SM = stage_min_blocks<T, N, true, TX * TY>();
     const bool wide = HAS_WIDE && c.sms > 0 && ctas <= WIDE_PER_SM * c.sms;
     if (prep) {
-        auto limit = [](auto k, size_t bytes) {
-            return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-        };
+        auto limit = [](auto k, size_t bytes) { return allow_smem(k, bytes); };
         cudaError_t e = limit(kern, smem);
         if (e == cudaSuccess && HAS_PF) e = limit(kern_pf, QUAD ? smem_q : smem);
         if (e == cudaSuccess && HAS_WIDE) e = limit(kern_w, smem);
@@ -270,7 +268,7 @@ static cudaError_t vjp_one(const LaunchCfg& c, const VjpPtrs& b, cudaStream_t s,
     }();
     const size_t smem = EQ == EQ_EULER ? sizeof(Quad<T>) * VjpQuadLayout<T, N, TX, TY>::TOTAL
                                        : sizeof(T) * VjpLayout<N, V, TX, TY>::TOTAL;
-    if (prep) return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (prep) return allow_smem(kern, smem);
     VjpArgs<T> A;
     A.q = static_cast<const T*>(b.q);
     A.rbar = static_cast<const T*>(b.rbar);
