@@ -55,17 +55,25 @@ __device__ __forceinline__ int fv_ghost(int i, int n, int transmissive)
     return i;
 }
 
-// Minmod of the slopes.  FP32: the minimum if both are positive plus the
-// maximum if both are negative.  FP64 (comparisons run on the FP64 pipe): one
-// comparison of the magnitudes and the signs from the high words.
+// Minmod of the slopes, zero where either is NaN (a face state next to a NaN
+// element takes no slope from it).  FP32: the minimum if both are positive plus
+// the maximum if both are negative; the inner pair passes a NaN on, the outer
+// one drops it.  FP64 (comparisons run on the FP64 pipe): one comparison of the
+// magnitudes, the signs and the NaN test from the high words (a difference that
+// is NaN is a quiet one).
 __device__ __forceinline__ float fv_minmod(float a, float b)
 {
-    return fmaxf(fminf(a, b), 0.f) + fminf(fmaxf(a, b), 0.f);
+    float lo, hi;
+    asm("min.NaN.f32 %0, %1, %2;" : "=f"(lo) : "f"(a), "f"(b));
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(hi) : "f"(a), "f"(b));
+    return fmaxf(lo, 0.f) + fminf(hi, 0.f);
 }
 __device__ __forceinline__ double fv_minmod(double a, double b)
 {
     const double m = ::fabs(a) < ::fabs(b) ? a : b;
-    return (__double2hiint(a) ^ __double2hiint(b)) < 0 ? 0.0 : m;
+    const int ha = __double2hiint(a), hb = __double2hiint(b);
+    const bool nan = max(ha & 0x7fffffff, hb & 0x7fffffff) > 0x7ff00000;
+    return (ha ^ hb) < 0 || nan ? 0.0 : m;
 }
 
 // The variables of one element.
