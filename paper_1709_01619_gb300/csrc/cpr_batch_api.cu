@@ -142,7 +142,7 @@ cudaError_t batch_launch(cpr_batch* b, Group& g, int fam, int grid, int mode, in
     B.swap = swap;
     B.tab = cpr::host_tab<T>(b->lcs[g.members[0]].tab);
     B.tp = cpr::host_tabpr<T>(b->lcs[g.members[0]].tab);
-    B.qx.tab = cpr::host_quadtab<T>(b->lcs[g.members[0]].tab, b->V == 1 || cpr::quad_joined<T>(g.p + 1));
+    B.qx.tab = cpr::host_quadtab<T>(b->lcs[g.members[0]].tab, cpr::quad_joined<T>(g.p + 1));
     const LaunchCfg& lc = b->lcs[g.members[0]];
     return fam == 0 ? cpr::batch_fam<T, 0>(g.p, lc.eqn, lc.flux, B, grid, s, 0, nullptr)
                     : cpr::batch_fam<T, 1>(g.p, lc.eqn, lc.flux, B, grid, s, 0, nullptr);
@@ -348,8 +348,9 @@ void fill_tables(cpr_batch* b, Group& g, const void* const* x)
             I.ntiles = I.tiles_x * ((lc.ny + ty - 1) / ty);
             I.tile0 = tile0;
             tile0 += I.ntiles;
-            I.rhx2 = T(2.0 / lc.hx);
-            I.rhy2 = T(2.0 / lc.hy);
+            // advection: the velocity in the factors (stage_tile_adv)
+            I.rhx2 = T(2.0 / lc.hx * (b->V == 1 ? lc.ax : 1.0));
+            I.rhy2 = T(2.0 / lc.hy * (b->V == 1 ? lc.ay : 1.0));
             I.ph.gamma = T(lc.gamma);
             I.ph.ax = T(lc.ax);
             I.ph.ay = T(lc.ay);

@@ -73,7 +73,7 @@ struct StageArgs {
     int mode;
     int do_avg, do_wave;
     int pf_lo;        // mode 6 on states larger than L2: launch the instantiation that prefetches the low part
-    T rhx2, rhy2;     // 2/hx, 2/hy
+    T rhx2, rhy2;     // 2/hx, 2/hy (CPR advection: times the velocity)
     Phys<T> ph;
     Tab<T> tab;
     TabPr<T> tp;      // the tables in pairs over points (two-lane path)

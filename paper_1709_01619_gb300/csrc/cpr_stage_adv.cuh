@@ -9,6 +9,9 @@
 // upwind edge state of the two faces: the upper edge of the lower element for
 // a >= 0, else the lower edge of the upper one.  Either way the state of face
 // f of a row of the tile is formed by one thread into slot f.
+// FP32 with N < 4 (quad_joined) takes D and the element's own edge states in
+// place of D', q_0 and q_{N-1}: every rounded entry of the operator is an error
+// common to all elements and steps, and there the joined one has more of it.
 //
 // Thread (el, k): row k of element el in phases 1 and 4, a column of an element
 // in phases 2 and 3.
@@ -61,6 +64,7 @@ __device__ __forceinline__ void stage_tile_adv(const StageArgs<T>& A, const Tab<
     T* yE = xE + L::XE;
     T* avS = yE + L::YE;
     const QuadTab<T>& qt = qx.tab;
+    constexpr bool J = quad_joined<T>(N);
     const int mode = A.mode;
     if (mode != MODE_RESIDUAL && A.ctrl->done) return;  // t_end reached: uniform exit
     // a limited run: clear the marked-element count of the limiter pass that
@@ -143,8 +147,8 @@ __device__ __forceinline__ void stage_tile_adv(const StageArgs<T>& A, const Tab<
         T c[N];
 #pragma unroll
         for (int b = 0; b < N; ++b) c[b] = sq[L::sq(elc, b, kc)];
-        c0 = c[0];
-        c1 = c[N - 1];
+        c0 = J ? c[0] : edge_lo<N>(qt, c);
+        c1 = J ? c[N - 1] : edge_hi<N>(qt, c);
         yE[L::ye(yup ? tyc + 1 : tyc, txc, kc)] = yup ? edge_hi<N>(qt, c) : edge_lo<N>(qt, c);
         if (A.bcy && yup && j0 + tyc == 0) yE[L::ye(0, txc, kc)] = edge_lo<N>(qt, c);
         if (A.bcy && !yup && j0 + tyc == A.ny - 1) yE[L::ye(TYe, txc, kc)] = edge_hi<N>(qt, c);
@@ -161,7 +165,8 @@ __device__ __forceinline__ void stage_tile_adv(const StageArgs<T>& A, const Tab<
     }
     T rx[N];
     if (valid) {
-        const T jl = xE[L::xe(ty, tx, k)] - x[0], jr = xE[L::xe(ty, tx + 1, k)] - x[N - 1];
+        const T jl = xE[L::xe(ty, tx, k)] - (J ? x[0] : edge_lo<N>(qt, x));
+        const T jr = xE[L::xe(ty, tx + 1, k)] - (J ? x[N - 1] : edge_hi<N>(qt, x));
         line_derivative<N>(qt, x, rx);
 #pragma unroll
         for (int a = 0; a < N; ++a) rx[a] = fma(jr, -qt.dgl[N - 1 - a], fma(jl, qt.dgl[a], rx[a]));
@@ -172,41 +177,47 @@ __device__ __forceinline__ void stage_tile_adv(const StageArgs<T>& A, const Tab<
     // ---- phase 4 ---------------------------------------------------------------
     T o[N];
     if (valid) {
-        // the factor of R in the stage's result
+        // R (2 / h here holds the velocity, rounded once), then the step: dt and
+        // the velocity rounded into one factor would be one more common error.
+        // FP32, 100 fixed steps on 48 x 45, mean error against 64 bits of eight
+        // states, in 1e-8, p = 1 / 2: 20.5 / 12.2 -> 18.1 / 8.6 without it, 11.8 / 6.9
+        // with the operator of N < 4 above (the general tile 12.0 / 9.8).
+#pragma unroll
+        for (int a = 0; a < N; ++a) o[a] = fma(-A.rhx2, rx[a], -A.rhy2 * sq[L::sq(el, k, a)]);
         T w = mode == MODE_RESIDUAL ? T(1) : T(A.ctrl->dt);
         if (mode == MODE_SO2 || mode == MODE_INC2) w *= T(0.25);
-        if (mode == MODE_SO3 || mode == MODE_INC3) w *= T(2.0 / 3.0);
-        const T sx = -A.rhx2 * A.ph.ax * w, sy = -A.rhy2 * A.ph.ay * w;
+        if (mode == MODE_INC1) {
 #pragma unroll
-        for (int a = 0; a < N; ++a) o[a] = fma(sx, rx[a], sy * sq[L::sq(el, k, a)]);
-        // the states last: few roundings of their size
-        if (mode == MODE_SO1 || mode == MODE_SO2 || mode == MODE_SO3) {
-            // (the smaller multiple first)
-            const T c0 = mode == MODE_SO2 ? T(0.25) : T(1.0 / 3.0);
-            const T c1 = mode == MODE_SO2 ? T(0.75) : T(2.0 / 3.0);
-            if (mode == MODE_SO1) {
+            for (int a = 0; a < N; ++a) o[a] *= w;
+        } else if (mode == MODE_SO1) {
 #pragma unroll
-                for (int a = 0; a < N; ++a) o[a] = x[a] + o[a];
-            } else {
-                T qn[N];
-                gload_row<N>(A.qn + off, qn);
+            for (int a = 0; a < N; ++a) o[a] = fma(w, o[a], x[a]);
+        } else if (mode == MODE_SO2 || mode == MODE_SO3) {
+            if (sizeof(T) == 8 && mode == MODE_SO3) w *= T(2.0 / 3.0);
+            T qn[N];
+            gload_row<N>(A.qn + off, qn);
 #pragma unroll
-                for (int a = 0; a < N; ++a)
-                    o[a] = fma(c1, mode == MODE_SO2 ? qn[a] : x[a], fma(c0, mode == MODE_SO2 ? x[a] : qn[a], o[a]));
+            for (int a = 0; a < N; ++a) {
+                if (mode == MODE_SO2) o[a] = fma(T(0.75), qn[a], fma(T(0.25), x[a], w * o[a]));
+                // FP32: as q + 2/3 ((q2 - q) + dt R), whose weights sum to one
+                // (stage_tile_quad)
+                else if (sizeof(T) == 4) o[a] = fma(T(2.0 / 3.0), fma(w, o[a], x[a] - qn[a]), qn[a]);
+                // (the smaller multiple first: its rounding is the smaller one)
+                else o[a] = fma(T(2.0 / 3.0), x[a], fma(T(1.0 / 3.0), qn[a], w * o[a]));
             }
         } else if (addb) {
             T b[N];
             gload_row<N>(A.qb + off, b);
             if (mode == MODE_INC2) {
 #pragma unroll
-                for (int a = 0; a < N; ++a) o[a] = fma(T(0.25), b[a], o[a]);
+                for (int a = 0; a < N; ++a) o[a] = fma(T(0.25), b[a], w * o[a]);
             } else {
                 T hi[N], lo[N];
                 gload_row<N>(A.qs + off, hi);
                 gload_row<N>(A.lo + off, lo);
 #pragma unroll
                 for (int a = 0; a < N; ++a) {
-                    compensated_add(hi[a], lo[a], fma(T(2.0 / 3.0), b[a], o[a]));
+                    compensated_add(hi[a], lo[a], T(2.0 / 3.0) * fma(w, o[a], b[a]));
                     o[a] = hi[a];
                 }
                 gstore_row<N>(A.lo + off, lo);

@@ -105,6 +105,8 @@ static cudaError_t stage_adv_tile(const LaunchCfg& c, StageArgs<T> A, cudaStream
     const size_t smem = stage_smem<T, P, EQ_ADV, TX, TY, false>();
     auto kern = cpr_stage_adv_kernel<T, P, TX, TY>;
     if (prep) return allow_smem(kern, smem);
+    A.rhx2 = T(2.0 / c.hx * c.ax);  // the operator's factors, the velocity in them
+    A.rhy2 = T(2.0 / c.hy * c.ay);
     A.tiles_x = (c.nx + TX - 1) / TX;
     div_magic((unsigned)A.tiles_x, &A.qx.tx_magic, &A.qx.tx_shift);
     kern<<<A.tiles_x * ((c.ny + TY - 1) / TY), stage_threads(TX * TY * (P + 1)), smem, s>>>(A);
@@ -227,7 +229,7 @@ static StageArgs<T> make_stage_args(const LaunchCfg& c, int mode, const StagePtr
     A.ph.ay = T(c.ay);
     A.tab = host_tab<T>(c.tab);
     A.tp = host_tabpr<T>(c.tab);
-    A.qx.tab = host_quadtab<T>(c.tab, c.eqn == EQ_ADV || (c.div == DIV_LP && quad_joined<T>(c.p + 1)));
+    A.qx.tab = host_quadtab<T>(c.tab, (c.eqn == EQ_ADV || c.div == DIV_LP) && quad_joined<T>(c.p + 1));
     div_magic((unsigned)A.tiles_x, &A.qx.tx_magic, &A.qx.tx_shift);
     return A;
 }
