@@ -1,4 +1,8 @@
-"""Rounding of the FP32 advection steps: the error of a run against the FP64
+"""Rounding of the FP32 steps.
+
+Shu-Osher stages of a vanishing step leave the state's bits alone.
+
+Advection: the error of a run against the FP64
 oracle is at most that of the same scheme written plainly in FP32 (flux
 derivative by the rows of D, edge values of the flux, corrections, the stages
 as compensated increments, each table entry and factor rounded once), on the
@@ -13,10 +17,11 @@ a few entries and factors, common to all states, and of many independent ones
 (thousands of values), so the ratio has no spread of that size."""
 import numpy as np
 import pytest
+import torch
 
 import oracle
 from paper_1709_01619_gb300 import _native as nat
-from test_gpu_parity import host, make, to_dev
+from test_gpu_parity import host, make, rough_state, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -84,3 +89,17 @@ def test_advection_error_at_most_the_plain_form(p):
             plain.append(np.linalg.norm(plain_run(c, q, steps, dt) - want) / norm)
     rms = [float(np.sqrt(np.mean(np.square(v)))) for v in (got, plain)]
     assert rms[0] <= 1.25 * rms[1], rms
+
+
+@pytest.mark.parametrize("eqn", [nat.EULER, nat.ADVECTION])
+@pytest.mark.parametrize("p", [1, 2, 3, 4])
+def test_stage_weights_sum_to_one(p, eqn):
+    """60 steps of size 1e-30 (every increment is far below the last place of
+    the state) with the limiter on (which marks nothing): the Shu-Osher stages
+    only average a state with itself, so its bits stay."""
+    c, o = make(nat.F32, eqn=eqn, nx=21, ny=13, p=p, x1=10.0, y1=6.0, limiter=1, tvb_M=1e9, lim_eps=1e-3, ax=0.7, ay=-0.4)
+    q = to_dev(rough_state(o, 3, noise=0.05), c)
+    with nat.Context(c) as ctx:
+        d = q.clone()
+        ctx.step(d, 60, 1e-30)
+    assert torch.equal(d, q)
