@@ -34,6 +34,8 @@
 // eight state arrays that a step has to move).
 #pragma once
 
+#include <algorithm>
+
 #include "cpr_common.cuh"
 #include "cpr_launch.h"
 #include "cpr_reduce.cuh"
@@ -43,7 +45,12 @@
 namespace cpr {
 
 constexpr int kFvCols = 28;   // columns of elements per warp
-constexpr int kFvWarps = 4;   // warps per CTA: neighbouring strips, whose rings overlap in L1
+// Warps per CTA.  FP32 four: neighbouring strips, whose rings overlap in L1.
+// FP64 one: the SM's FP64 pipe is busy from four warps on, however they share
+// CTAs, so single warps spread a grid most evenly (256^2 second order, Euler /
+// Roe: 45.7 / 98.8 us a residual with four, 37.3 / 76.2 with one).
+template <class T>
+constexpr int kFvWarps = sizeof(T) == 8 ? 1 : 4;
 
 // Wrapped (periodic) or clamped (transmissive) element index, for indices
 // at most two outside [0, n) (no integer division: n may be 1).
@@ -176,7 +183,7 @@ constexpr int fv_min_blocks()
 
 // MODE: the stage mode, or -1 for the one in the arguments.
 template <class T, int EQ, int FLUX, int ORDER, int MODE>
-__global__ void __launch_bounds__(kFvWarps * 32, fv_min_blocks<T>())
+__global__ void __launch_bounds__(kFvWarps<T> * 32, fv_min_blocks<T>())
 cpr_fv_stage_kernel(const StageArgs<T> A, const int rows)
 {
     constexpr int V = NVars<EQ>::value;
@@ -186,7 +193,7 @@ cpr_fv_stage_kernel(const StageArgs<T> A, const int rows)
     const int lane = threadIdx.x & 31;
     // rows by CTA, so that every row pointer is uniform over the CTA
     const int by = blockIdx.x / A.tiles_x, j0 = by * rows, jend = min(j0 + rows, A.ny);
-    const int i0 = ((blockIdx.x - by * A.tiles_x) * kFvWarps + (threadIdx.x >> 5)) * kFvCols;
+    const int i0 = ((blockIdx.x - by * A.tiles_x) * kFvWarps<T> + (threadIdx.x >> 5)) * kFvCols;
     const int col = i0 + lane - 2;
     const bool valid = lane >= 2 && lane < 2 + kFvCols && col < A.nx;
     const bool addb = mode == MODE_INC2 || mode == MODE_INC3;
@@ -245,39 +252,43 @@ cpr_fv_stage_kernel(const StageArgs<T> A, const int rows)
             fv_states<ORDER>(d, dyn, dnn, up, dn);
             const El Ghi = fv_face2<EQ, FLUX, 1>(upl, dn, A.ph);
             upl = up;
-            // left face, and the right one from the next lane
-            const El dx = fv_diff(c, fv_up_lane(c));
-            fv_states<ORDER>(c, dx, fv_down_lane(dx), up, dn);
-            const El Fl = fv_face2<EQ, FLUX, 0>(fv_up_lane(up), dn, A.ph);
-            El o = fv_scale(sx, fv_diff(fv_down_lane(Fl), Fl));
-            // (the step's factor last: rounded into sx and sy it would be an
-            // error common to every element and step, which does not average out)
-            o = fv_scale(w, fv_axpy(sy, fv_diff(Ghi, Glo), o));
-            if (mode == MODE_SO1) {
-                o = fv_axpy(T(1), s0, o);
-            } else if (mode == MODE_SO2 || mode == MODE_SO3) {
-                o = fv_axpy(mode == MODE_SO2 ? T(0.75) : T(1.0 / 3.0), s1,
-                            fv_axpy(mode == MODE_SO2 ? T(0.25) : T(2.0 / 3.0), s0, o));
-            } else if (mode == MODE_INC2) {
-                o = fv_axpy(T(0.25), s0, o);
-            } else if (mode == MODE_INC3) {
-                o = fv_axpy(T(2.0 / 3.0), s1, o);
+            // FP64: no x-faces of the row below the strip, on the pipe that bounds
+            // the kernel (FP32 third order measured 4 % slower with the branch)
+            if (sizeof(T) == 4 || j >= j0) {
+                // left face, and the right one from the next lane
+                const El dx = fv_diff(c, fv_up_lane(c));
+                fv_states<ORDER>(c, dx, fv_down_lane(dx), up, dn);
+                const El Fl = fv_face2<EQ, FLUX, 0>(fv_up_lane(up), dn, A.ph);
+                El o = fv_scale(sx, fv_diff(fv_down_lane(Fl), Fl));
+                // (the step's factor last: rounded into sx and sy it would be an
+                // error common to every element and step, which does not average out)
+                o = fv_scale(w, fv_axpy(sy, fv_diff(Ghi, Glo), o));
+                if (mode == MODE_SO1) {
+                    o = fv_axpy(T(1), s0, o);
+                } else if (mode == MODE_SO2 || mode == MODE_SO3) {
+                    o = fv_axpy(mode == MODE_SO2 ? T(0.75) : T(1.0 / 3.0), s1,
+                                fv_axpy(mode == MODE_SO2 ? T(0.25) : T(2.0 / 3.0), s0, o));
+                } else if (mode == MODE_INC2) {
+                    o = fv_axpy(T(0.25), s0, o);
+                } else if (mode == MODE_INC3) {
+                    o = fv_axpy(T(2.0 / 3.0), s1, o);
 #pragma unroll
-                for (int v = 0; v < V; ++v) {
-                    compensated_add(s0.v[v], s2.v[v], o.v[v]);
-                    o.v[v] = s0.v[v];
+                    for (int v = 0; v < V; ++v) {
+                        compensated_add(s0.v[v], s2.v[v], o.v[v]);
+                        o.v[v] = s0.v[v];
+                    }
                 }
-            }
-            if (valid && j >= j0) {
-                const long long r0 = (long long)j * A.nx;
+                if (valid && j >= j0) {
+                    const long long r0 = (long long)j * A.nx;
 #pragma unroll
-                for (int v = 0; v < V; ++v) {
-                    (A.out + v * A.npts + r0)[gi] = o.v[v];
-                    if (mode == MODE_INC3) (A.lo + v * A.npts + r0)[gi] = s2.v[v];
-                }
-                if (A.do_wave) {
-                    const T sp = point_speed<EQ, true>(o.v, A.ph);
-                    m = sp > m ? sp : m;
+                    for (int v = 0; v < V; ++v) {
+                        (A.out + v * A.npts + r0)[gi] = o.v[v];
+                        if (mode == MODE_INC3) (A.lo + v * A.npts + r0)[gi] = s2.v[v];
+                    }
+                    if (A.do_wave) {
+                        const T sp = point_speed<EQ, true>(o.v, A.ph);
+                        m = sp > m ? sp : m;
+                    }
                 }
             }
             c = d;
@@ -289,22 +300,36 @@ cpr_fv_stage_kernel(const StageArgs<T> A, const int rows)
     if (A.do_wave) block_time_update<T>(m, A.ctrl, /*advance=*/true, gridDim.x);
 }
 
-// Rows per strip: a strip costs about two rows beyond its own, and the pass
-// takes the time of the SM with most CTAs; a row takes 0.6 us plus 0.14 us for
-// every CTA that shares its SM, so few tall strips leave the SM waiting.  Of
-// the heights that give every SM almost its resident CTAs or more, the one with
-// the fewest rows on the busiest SM (1536^2: 24 rows, six CTAs each; 37 us per
-// stage, 36 rows and four CTAs 50); smaller grids take two rows.
+// Rows per strip.
+//
+// FP32: a strip costs about two rows beyond its own, and the pass takes the time
+// of the SM with most CTAs; a row takes 0.6 us plus 0.14 us for every CTA that
+// shares its SM, so few tall strips leave the SM waiting.  Of the heights that
+// give every SM almost its resident CTAs or more, the one with the fewest rows
+// on the busiest SM (1536^2: 24 rows, six CTAs each; 37 us per stage, 36 rows and
+// four CTAs 50); smaller grids take two rows.
+//
+// FP64: the pass takes the time of the busiest SM's rows (1.45 us for a
+// second-order Euler row of one warp); up to four warps take the time of 4.5,
+// and a strip costs half a row beyond its own (the y-face below it).  Of heights
+// 1, 2, 3, ..., 8, 10, ..., 32 on fourteen grids from 32^2 to 1536^2, every order,
+// flux and equation, this choice is 1 % from the fastest on average, 9 % at worst,
+// and never slower than a tile of 32 x 8 elements.  us a residual, second order,
+// that tile -> FP32's rule and CTAs -> these: Euler 192^2 37 -> 41 -> 25, 512^2
+// 180 -> 148 -> 114, 1536^2 1515 -> 891 -> 844; Roe 192^2 58 -> 85 -> 51, 512^2
+// 300 -> 319 -> 251.
+template <class T>
 inline int fv_rows(int ctas_x, int ny, int sms)
 {
-    constexpr int kMaxRows = 48;
-    int best = 2;
-    long long cost = -1;
-    for (int r = 2; r <= kMaxRows; ++r) {
-        const long long ctas = (long long)ctas_x * ((ny + r - 1) / r);
-        if (r > 2 && ctas < (long long)(kFvResident - 1) * sms) break;
-        const long long c = (ctas + sms - 1) / sms * (r + 2);
-        if (cost < 0 || c <= cost) {
+    constexpr bool F64 = sizeof(T) == 8;
+    constexpr int kMaxRows = F64 ? 32 : 48;
+    int best = 0;
+    long long cost = 0;
+    for (int r = F64 ? 1 : 2; r <= kMaxRows; ++r) {
+        const long long ctas = (long long)ctas_x * ((ny + r - 1) / r), per_sm = (ctas + sms - 1) / sms;
+        if (!F64 && r > 2 && ctas < (long long)(kFvResident - 1) * sms) break;
+        const long long c = F64 ? std::max(2 * per_sm, 9LL) * (2 * r + 1) : per_sm * (r + 2);
+        if (best == 0 || c <= cost) {
             best = r;
             cost = c;
         }
@@ -315,10 +340,10 @@ inline int fv_rows(int ctas_x, int ny, int sms)
 template <class T, int EQ, int FLUX, int ORDER>
 static cudaError_t fv_order(const LaunchCfg& c, const StageArgs<T>& A, cudaStream_t s)
 {
-    const int rows = fv_rows(A.tiles_x, c.ny, c.sms > 0 ? c.sms : 1);
+    const int rows = fv_rows<T>(A.tiles_x, c.ny, c.sms > 0 ? c.sms : 1);
     const int ctas = A.tiles_x * ((c.ny + rows - 1) / rows);
     auto launch = [&](auto k) {
-        k<<<ctas, kFvWarps * 32, 0, s>>>(A, rows);
+        k<<<ctas, kFvWarps<T> * 32, 0, s>>>(A, rows);
         return cudaGetLastError();
     };
     // FP32 steps take a kernel compiled for their stage mode

@@ -11,7 +11,7 @@ template <class T>
 cudaError_t launch_fv(const LaunchCfg& c, int mode, const StagePtrs& b, bool do_wave, cudaStream_t s)
 {
     StageArgs<T> A = make_stage_args<T>(c, mode, b, do_wave);
-    A.tiles_x = (c.nx + kFvCols * kFvWarps - 1) / (kFvCols * kFvWarps);
+    A.tiles_x = (c.nx + kFvCols * kFvWarps<T> - 1) / (kFvCols * kFvWarps<T>);
     A.do_avg = 0;  // FV runs have no troubled-cell limiter, hence no averages pass
     if (c.eqn == EQ_EULER)
         return c.flux == FLUX_ROE ? fv_one<T, EQ_EULER, FLUX_ROE>(c, A, s) : fv_one<T, EQ_EULER, FLUX_RUSANOV>(c, A, s);
