@@ -35,6 +35,7 @@
 #pragma once
 
 #include <algorithm>
+#include <type_traits>
 
 #include "cpr_common.cuh"
 #include "cpr_launch.h"
@@ -181,6 +182,41 @@ constexpr int fv_min_blocks()
     return sizeof(T) == 4 ? kFvResident : 1;
 }
 
+// What the stage update adds to a row (row_of reads a row of an array).
+template <class T, class El, class F>
+__device__ __forceinline__ void fv_terms(int mode, const StageArgs<T>& A, int j, F&& row_of, El& s0, El& s1, El& s2)
+{
+    if (mode >= MODE_SO1 && mode != MODE_INC1) s0 = row_of(mode == MODE_INC2 ? A.qb : A.qs, j);
+    if (mode == MODE_SO2 || mode == MODE_SO3) s1 = row_of(A.qn, j);
+    if (mode == MODE_INC3) {
+        s1 = row_of(A.qb, j);
+        s2 = row_of(A.lo, j);
+    }
+}
+
+// The stage's result from o, R times the step's factor of the stage.
+template <class T, int V>
+__device__ __forceinline__ FvEl<T, V> fv_update(int mode, FvEl<T, V> o, FvEl<T, V> s0, const FvEl<T, V>& s1,
+                                                FvEl<T, V>& s2)
+{
+    if (mode == MODE_SO1) {
+        o = fv_axpy(T(1), s0, o);
+    } else if (mode == MODE_SO2 || mode == MODE_SO3) {
+        o = fv_axpy(mode == MODE_SO2 ? T(0.75) : T(1.0 / 3.0), s1,
+                    fv_axpy(mode == MODE_SO2 ? T(0.25) : T(2.0 / 3.0), s0, o));
+    } else if (mode == MODE_INC2) {
+        o = fv_axpy(T(0.25), s0, o);
+    } else if (mode == MODE_INC3) {
+        o = fv_axpy(T(2.0 / 3.0), s1, o);
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+            compensated_add(s0.v[v], s2.v[v], o.v[v]);
+            o.v[v] = s0.v[v];
+        }
+    }
+    return o;
+}
+
 // MODE: the stage mode, or -1 for the one in the arguments.
 template <class T, int EQ, int FLUX, int ORDER, int MODE>
 __global__ void __launch_bounds__(kFvWarps<T> * 32, fv_min_blocks<T>())
@@ -236,17 +272,16 @@ cpr_fv_stage_kernel(const StageArgs<T> A, const int rows)
         const T sx = T(-0.25) * A.rhx2, sy = T(-0.25) * A.rhy2;
         // row j0 - 1 is there for its upper face only (the same instructions
         // for every face, so that both warps of a face see the same bits)
-        for (int j = j0 - 1; j < jend; ++j) {
+        // (FP32 counts from zero: the third-order Euler kernel spills otherwise,
+        // 1536^2 1.614 -> 1.583 ms for 12 steps; FP64 takes fewer registers with j)
+        const int first = sizeof(T) == 4 ? j0 - 1 : 0;
+        for (int k = j0 - 1 - first; first + k < jend; ++k) {
+            const int j = first + k;
             const El n = row();  // row j + 2
             if (j + 1 < jend) fetch(j + 3);
             const int jo = max(j, j0);
             El s0, s1, s2;  // what the stage update adds: started here, used last
-            if (mode >= MODE_SO1 && mode != MODE_INC1) s0 = row_of(mode == MODE_INC2 ? A.qb : A.qs, jo);
-            if (mode == MODE_SO2 || mode == MODE_SO3) s1 = row_of(A.qn, jo);
-            if (mode == MODE_INC3) {
-                s1 = row_of(A.qb, jo);
-                s2 = row_of(A.lo, jo);
-            }
+            fv_terms(mode, A, jo, row_of, s0, s1, s2);
             // upper face of the row
             const El dnn = fv_diff(n, d);
             fv_states<ORDER>(d, dyn, dnn, up, dn);
@@ -263,21 +298,7 @@ cpr_fv_stage_kernel(const StageArgs<T> A, const int rows)
                 // (the step's factor last: rounded into sx and sy it would be an
                 // error common to every element and step, which does not average out)
                 o = fv_scale(w, fv_axpy(sy, fv_diff(Ghi, Glo), o));
-                if (mode == MODE_SO1) {
-                    o = fv_axpy(T(1), s0, o);
-                } else if (mode == MODE_SO2 || mode == MODE_SO3) {
-                    o = fv_axpy(mode == MODE_SO2 ? T(0.75) : T(1.0 / 3.0), s1,
-                                fv_axpy(mode == MODE_SO2 ? T(0.25) : T(2.0 / 3.0), s0, o));
-                } else if (mode == MODE_INC2) {
-                    o = fv_axpy(T(0.25), s0, o);
-                } else if (mode == MODE_INC3) {
-                    o = fv_axpy(T(2.0 / 3.0), s1, o);
-#pragma unroll
-                    for (int v = 0; v < V; ++v) {
-                        compensated_add(s0.v[v], s2.v[v], o.v[v]);
-                        o.v[v] = s0.v[v];
-                    }
-                }
+                o = fv_update(mode, o, s0, s1, s2);
                 if (valid && j >= j0) {
                     const long long r0 = (long long)j * A.nx;
 #pragma unroll
@@ -298,6 +319,89 @@ cpr_fv_stage_kernel(const StageArgs<T> A, const int rows)
         }
     }
     if (A.do_wave) block_time_update<T>(m, A.ctrl, /*advance=*/true, gridDim.x);
+}
+
+// Strips of two rows of one FP32 variable (advection): every load first, so that
+// a strip takes one latency of L2 where the walk above takes one per row, which
+// is most of a small grid's time.  The end-of-run flag is tested where something
+// is written (an exit before the loads are used would wait for it ahead of
+// them), and the registers are bounded as the walk's (unbounded, the compiler
+// settles for 32 to 40 and fewer loads in flight: 64^2 3.7).  us per stage, second
+// order, tiles of 32 x 8 elements -> walk -> this: 64^2 4.1 -> 4.3 -> 3.0, 160^2
+// 4.0 -> 4.8 -> 3.1, 400^2 5.5 -> 5.4 -> 3.9.
+constexpr int kFvShort = 2;
+template <class T, int EQ>
+constexpr bool fv_has_short = sizeof(T) == 4 && EQ == EQ_ADV;
+
+template <class T, int EQ, int FLUX, int ORDER, int MODE>
+__global__ void __launch_bounds__(kFvWarps<T> * 32, fv_min_blocks<T>()) cpr_fv_short_kernel(const StageArgs<T> A)
+{
+    constexpr int V = NVars<EQ>::value, R = kFvShort;
+    using El = FvEl<T, V>;
+    const int mode = MODE >= 0 ? MODE : A.mode;
+    const bool done = mode > 0 && A.ctrl->done;  // t_end reached (uniform over the grid)
+    const int lane = threadIdx.x & 31;
+    const int by = blockIdx.x / A.tiles_x, j0 = by * R;
+    const int i0 = ((blockIdx.x - by * A.tiles_x) * kFvWarps<T> + (threadIdx.x >> 5)) * kFvCols;
+    const int col = i0 + lane - 2;
+    const bool valid = lane >= 2 && lane < 2 + kFvCols && col < A.nx;
+    const bool addb = mode == MODE_INC2 || mode == MODE_INC3;
+    const unsigned int gi = (unsigned int)fv_ghost(min(col, A.nx + 1), A.nx, A.bcx);
+    T m = T(0);
+
+    if (i0 < A.nx) {
+        auto row_of = [&](const T* p, int j) {
+            El x;
+            p += (long long)j * A.nx;
+#pragma unroll
+            for (int v = 0; v < V; ++v) x.v[v] = (p + v * A.npts)[gi];
+            return x;
+        };
+        El x[R + 4], b[R + 4], s0[R], s1[R], s2[R];  // rows j0 - 2 .. j0 + R + 1; terms of the update
+#pragma unroll
+        for (int k = 0; k < R + 4; ++k) {
+            const int j = fv_ghost(j0 - 2 + k, A.ny, A.bcy);
+            x[k] = row_of(A.qs, j);
+            if (addb) b[k] = row_of(A.qb, j);
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) fv_terms(mode, A, min(j0 + r, A.ny - 1), row_of, s0[r], s1[r], s2[r]);
+#pragma unroll
+        for (int k = 0; k < R + 4; ++k)
+            if (addb) x[k] = fv_axpy(T(1), x[k], b[k]);
+        El G[R + 1], up[R + 2], dn[R + 2];  // flux of the lower face, states along y of row j0 - 1 + k
+#pragma unroll
+        for (int k = 0; k < R + 2; ++k)
+            fv_states<ORDER>(x[k + 1], fv_diff(x[k + 1], x[k]), fv_diff(x[k + 2], x[k + 1]), up[k], dn[k]);
+#pragma unroll
+        for (int k = 0; k <= R; ++k) G[k] = fv_face2<EQ, FLUX, 1>(up[k], dn[k + 1], A.ph);
+        T w = mode > 0 ? T(A.ctrl->dt) : T(1);
+        if (mode == MODE_SO2 || mode == MODE_INC2) w *= T(0.25);
+        if (mode == MODE_SO3 || mode == MODE_INC3) w *= T(2.0 / 3.0);
+        const T sx = T(-0.25) * A.rhx2, sy = T(-0.25) * A.rhy2;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const El c = x[r + 2], dx = fv_diff(c, fv_up_lane(c));
+            El xu, xd;
+            fv_states<ORDER>(c, dx, fv_down_lane(dx), xu, xd);
+            const El Fl = fv_face2<EQ, FLUX, 0>(fv_up_lane(xu), xd, A.ph);
+            El o = fv_scale(sx, fv_diff(fv_down_lane(Fl), Fl));
+            o = fv_update(mode, fv_scale(w, fv_axpy(sy, fv_diff(G[r + 1], G[r]), o)), s0[r], s1[r], s2[r]);
+            if (valid && !done && j0 + r < A.ny) {
+                const long long r0 = (long long)(j0 + r) * A.nx;
+#pragma unroll
+                for (int v = 0; v < V; ++v) {
+                    (A.out + v * A.npts + r0)[gi] = o.v[v];
+                    if (mode == MODE_INC3) (A.lo + v * A.npts + r0)[gi] = s2[r].v[v];
+                }
+                if (A.do_wave) {
+                    const T sp = point_speed<EQ, true>(o.v, A.ph);
+                    m = sp > m ? sp : m;
+                }
+            }
+        }
+    }
+    if (A.do_wave && !done) block_time_update<T>(m, A.ctrl, /*advance=*/true, gridDim.x);
 }
 
 // Rows per strip.
@@ -342,17 +446,24 @@ static cudaError_t fv_order(const LaunchCfg& c, const StageArgs<T>& A, cudaStrea
 {
     const int rows = fv_rows<T>(A.tiles_x, c.ny, c.sms > 0 ? c.sms : 1);
     const int ctas = A.tiles_x * ((c.ny + rows - 1) / rows);
-    auto launch = [&](auto k) {
-        k<<<ctas, kFvWarps<T> * 32, 0, s>>>(A, rows);
+    auto launch = [&](auto m) {
+        constexpr int M = decltype(m)::value;
+        if constexpr (fv_has_short<T, EQ>) {
+            if (rows == kFvShort) {
+                cpr_fv_short_kernel<T, EQ, FLUX, ORDER, M><<<ctas, kFvWarps<T> * 32, 0, s>>>(A);
+                return cudaGetLastError();
+            }
+        }
+        cpr_fv_stage_kernel<T, EQ, FLUX, ORDER, M><<<ctas, kFvWarps<T> * 32, 0, s>>>(A, rows);
         return cudaGetLastError();
     };
     // FP32 steps take a kernel compiled for their stage mode
     if constexpr (sizeof(T) == 4) {
-        if (A.mode == MODE_INC1) return launch(cpr_fv_stage_kernel<T, EQ, FLUX, ORDER, MODE_INC1>);
-        if (A.mode == MODE_INC2) return launch(cpr_fv_stage_kernel<T, EQ, FLUX, ORDER, MODE_INC2>);
-        if (A.mode == MODE_INC3) return launch(cpr_fv_stage_kernel<T, EQ, FLUX, ORDER, MODE_INC3>);
+        if (A.mode == MODE_INC1) return launch(std::integral_constant<int, MODE_INC1>{});
+        if (A.mode == MODE_INC2) return launch(std::integral_constant<int, MODE_INC2>{});
+        if (A.mode == MODE_INC3) return launch(std::integral_constant<int, MODE_INC3>{});
     }
-    return launch(cpr_fv_stage_kernel<T, EQ, FLUX, ORDER, -1>);
+    return launch(std::integral_constant<int, -1>{});
 }
 
 template <class T, int EQ, int FLUX>

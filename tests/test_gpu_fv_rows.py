@@ -7,6 +7,7 @@ against the FP64 oracle: residual, and two fixed steps.
 Tolerances: those of the other FV comparisons (FP64 1e-12, FP32 residual 1e-5,
 steps 1e-6)."""
 import pytest
+import torch
 
 import oracle
 from paper_1709_01619_gb300 import _native as nat
@@ -36,3 +37,21 @@ def test_strip_heights(eqn, flux, size, dtype, scheme):
         assert rel(host(ctx.residual(d)), R_or) <= (TOL64 if dtype == nat.F64 else TOL32)
         ctx.step(d, 2, 1e-4)
         assert rel(host(d), q_or) <= (TOL64 if dtype == nat.F64 else 1e-6)
+
+
+@pytest.mark.parametrize("eqn", [nat.EULER, nat.ADVECTION])
+@pytest.mark.parametrize("dtype", [nat.F64, nat.F32])
+@pytest.mark.parametrize("size", [(100, 99), (30, 700)])
+def test_steps_after_the_end_change_nothing(eqn, dtype, size):
+    """A run ends in its fourth step, shortened; the launches of further steps
+    leave the state, in whichever buffer it is."""
+    c, o = make(dtype, eqn=eqn, nx=size[0], ny=size[1], x1=10.0, y1=10.0, ax=0.7, ay=-1.2)
+    q = state(o, "vortex", 3)
+    runs = []
+    for steps in (4, 5, 40):
+        with nat.Context(c) as ctx:
+            d = dev(q, c)
+            ctx.step(d, steps, 1e-3, 3.5e-3)
+            assert ctx.get_time() == (3.5e-3, 4)
+            runs.append(d)
+    assert torch.equal(runs[0], runs[1]) and torch.equal(runs[0], runs[2])
