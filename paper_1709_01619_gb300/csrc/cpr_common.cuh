@@ -94,9 +94,9 @@ struct Phys {
     T ax, ay; // advection
 };
 
-// Reciprocal and square root in the FP32 physics (1/rho, sound speed): the
+// Reciprocal and square root of the physics (1/rho, sound speed).  FP32: the
 // hardware approximations (a few ulp), at the level of the rounding of the
-// flux itself.  FP64 keeps IEEE operations.
+// flux itself; FP64: the IEEE operations.
 __device__ __forceinline__ float frcp(float x) { return __fdividef(1.0f, x); }
 __device__ __forceinline__ double frcp(double x) { return 1.0 / x; }
 __device__ __forceinline__ float fsqrt(float x)
@@ -105,11 +105,12 @@ __device__ __forceinline__ float fsqrt(float x)
     return x >= 0.0f ? x * rsqrtf(fmaxf(x, 1.17549435e-38f)) : __int_as_float(0x7fffffff);
 }
 __device__ __forceinline__ double fsqrt(double x) { return sqrt(x); }
-// The same as single instructions (1 ulp and 2^-23; flush-to-zero forms, which
-// leave out the scaling of subnormal operands), for the stage updates (FTZ in
-// the physics below).  The stand-alone FP32 residual keeps the forms above:
-// its relative rounding is that of O(1) fluxes over a small result, so any
-// other rounding would show in it.
+// The forms of the stage updates (FTZ in the physics below).  FP32: the single
+// instructions (1 ulp and 2^-23; flush-to-zero forms, which leave out the
+// scaling of subnormal operands).  The stand-alone FP32 residual of the CPR
+// schemes keeps the forms above: its relative rounding is that of O(1) fluxes
+// over a small result, so any other rounding would show in it.  (The FV residual
+// takes these; its error is the same with either.)
 __device__ __forceinline__ float frcp_ftz(float x)
 {
     float r;
@@ -122,14 +123,19 @@ __device__ __forceinline__ float fsqrt_ftz(float x)
     asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
-// In FP64, where an operation keeps a scheduler busy for 64 cycles: the ~20-bit
-// hardware seed y and one third-order correction from the residual e, the
-// binomial series of (1 - e)^-1 and (1 - e)^-1/2 cut after e^2 (Householder's
-// method of order 2; the next term is below 2^-57):
-//   1/x = y (1 + e + e^2), e = 1 - x y;
-//   sqrt(x) = s (1 + e/2 + 3 e^2/8), s = x y, e = 1 - s y.
-// Three and five operations.  Zeros, infinities and NaN keep the IEEE results
-// (tested on the bits, off the FP64 pipe); subnormal operands count as zero.
+// FP64 (every Euler kernel but the norms), where an operation keeps a scheduler
+// busy for 64 cycles: from the ~20-bit hardware seed y in three and five
+// operations.
+//   1/x: the geometric series of (1 - e)^-1 cut after e^2, y (1 + e + e^2) with
+//     e = 1 - x y; e^3 < 2^-58 is left.
+//   sqrt(x): Newton's step for s = x y, g = s + s (1/2 - h s) with h = y / 2,
+//     then one step of Heron's method from the exact residual, g + h (x - g^2).
+//     Newton's step leaves 2^-38, times the 2^-19 of h.
+// Both round within 0.55 units of the last place (a series for the root like
+// the reciprocal's, as many operations, within 0.8).  Zeros, infinities, NaN
+// and negative operands give the IEEE results (tested on the bits, off the FP64
+// pipe); subnormal operands count as zero (the root returns the operand), and
+// so do reciprocals below the normal range.
 __device__ __forceinline__ double frcp_ftz(double x)
 {
     double y;
@@ -143,10 +149,13 @@ __device__ __forceinline__ double fsqrt_ftz(double x)
 {
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double s = x * y, e = fma(-s, y, 1.0);
-    const double r = fma(s, fma(0.375, e, 0.5) * e, s);
-    const unsigned int h = (unsigned int)__double2hiint(x);
-    return h - 0x00100000u >= 0x7fe00000u && h <= 0x80000000u ? x : r;
+    // y / 2 by the exponent (y of a normal positive x is normal)
+    const double h = __hiloint2double(__double2hiint(y) - 0x00100000, __double2loint(y));
+    const double s = x * y, g = fma(s, fma(-h, s, 0.5), s);
+    const double r = fma(h, fma(-g, g, x), g);
+    const unsigned int hx = (unsigned int)__double2hiint(x);
+    if (hx - 0x00100000u < 0x7fe00000u) return r;
+    return hx > 0x80000000u ? __hiloint2double(0x7fffffff, -1) : x;
 }
 template <bool FTZ, class T>
 __device__ __forceinline__ T rcp_of(T x)
