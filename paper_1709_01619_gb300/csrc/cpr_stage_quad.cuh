@@ -630,13 +630,18 @@ __device__ __forceinline__ void stage_tile_quad(const StageArgs<float>& A, const
 }
 
 // Resident CTAs per SM of a single problem's kernels.  p = 4: 4 CTAs of 32
-// elements (94 registers, no spills) instead of the 6 (64 registers, 44 bytes
+// elements (96 registers, no spills) instead of the 6 (64 registers, 56 bytes
 // of spills) that batches keep: 821 x 819 p = 4 303 -> 281 us per stage, the
-// 64-instance batch 31.5 -> 32.5 ms per 24 steps.
+// 64-instance batch 31.5 -> 32.5 ms per 24 steps.  p = 1: 7 CTAs (72 registers,
+// which LP with Rusanov's flux takes anyway) for every grid; with the 76 to 85 of
+// the other divergences and fluxes, grids around 256^2 need a second round of
+// CTAs: Roe 10.6 -> 8.2 us per stage (the general tile 10.1), 768^2 57.7 -> 52.7.
 template <int P, bool WIDE, int ELEMS>
 constexpr int quad_min_blocks()
 {
-    return P == 4 && !WIDE ? 128 / ELEMS : stage_min_blocks<float, P + 1, WIDE, ELEMS>();
+    return P == 1             ? 7 * 64 / ELEMS
+           : P == 4 && !WIDE ? 128 / ELEMS
+                             : stage_min_blocks<float, P + 1, WIDE, ELEMS>();
 }
 
 // The kernels that the step adjoint launches behind one another: those compiled

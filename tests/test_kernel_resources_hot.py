@@ -31,18 +31,18 @@ def resident(regs, threads):
 
 
 # resident CTAs per SM of the kernels for large grids of one problem, and threads per CTA
-QUAD = {1: (4, 128), 2: (6, 192), 3: (4, 256), 4: (4, 160)}
+QUAD = {1: (7, 128), 2: (6, 192), 3: (4, 256), 4: (4, 160)}
 
 
 @pytest.mark.parametrize("p", [1, 2, 3, 4])
 def test_fp32_euler_stages(p):
     """cpr_stage_quad_kernel<P, DIV, FLUX, TX, TY, MINB, MODE>: for LP and Rusanov
     one kernel per stage mode, in a form for large grids and one for two CTAs per
-    SM (p = 4: the same), none of which spills; the kernels for every mode
+    SM (p = 1 and 4: the same), none of which spills; the kernels for every mode
     (other divergences and fluxes, mode 0) spill only in the forms for large grids
     of p = 2 and 3, at most 48 bytes."""
     ctas, threads = QUAD[p]
-    wide = ctas if p == 4 else 2
+    wide = ctas if p in (1, 4) else 2
     q = kernels(f"cpr_stage_f32_p{p}.cu", "cpr_stage_quad_kernel")
     modes = {}
     for (_, div, flux, _, _, minb, mode), r in q.items():
