@@ -512,7 +512,9 @@ extern "C" cpr_status cpr_batch_init(const cpr_config* cfgs, int n, void* stream
     for (int i = 0; i < n && e == cudaSuccess; ++i) {
         b->lcs[i].ctrl = b->ctrls + i;
     }
-    // order groups
+    // order groups: instances of one order share the operator tables of the first
+    // (on Gauss points, the only ones of a batch, every correction has the same
+    // tables, to 1e-14)
     for (int p = 1; p <= 4 && e == cudaSuccess; ++p) {
         Group g;
         g.p = p;
