@@ -190,55 +190,45 @@ __device__ __forceinline__ T pressure(const T* q, T gamma, T& u, T& v)
     return pressure(q, gamma, u, v, r);
 }
 
-// x-flux f(q) and y-flux g(q) of Eq. 4.
+// x-flux f(q) and y-flux g(q) of Eq. 4 (Euler).
 template <int EQ, class T>
 __device__ __forceinline__ void flux_x(const T* q, const Phys<T>& ph, T* f)
 {
-    if constexpr (EQ == EQ_ADV) {
-        f[0] = ph.ax * q[0];
-    } else {
-        T u, v;
-        T p = pressure(q, ph.gamma, u, v);
-        f[0] = q[1];
-        f[1] = q[1] * u + p;
-        f[2] = q[2] * u;
-        f[3] = (q[3] + p) * u;
-    }
+    static_assert(EQ == EQ_EULER, "advection kernels need no point flux");
+    T u, v;
+    T p = pressure(q, ph.gamma, u, v);
+    f[0] = q[1];
+    f[1] = q[1] * u + p;
+    f[2] = q[2] * u;
+    f[3] = (q[3] + p) * u;
 }
-
 template <int EQ, class T>
 __device__ __forceinline__ void flux_y(const T* q, const Phys<T>& ph, T* g)
 {
-    if constexpr (EQ == EQ_ADV) {
-        g[0] = ph.ay * q[0];
-    } else {
-        T u, v;
-        T p = pressure(q, ph.gamma, u, v);
-        g[0] = q[2];
-        g[1] = q[1] * v;
-        g[2] = q[2] * v + p;
-        g[3] = (q[3] + p) * v;
-    }
+    static_assert(EQ == EQ_EULER, "advection kernels need no point flux");
+    T u, v;
+    T p = pressure(q, ph.gamma, u, v);
+    g[0] = q[2];
+    g[1] = q[1] * v;
+    g[2] = q[2] * v + p;
+    g[3] = (q[3] + p) * v;
 }
 
 // Directional derivative of the x- or y-flux, A(q) dq (the chain-rule
-// divergence of Sec. 2.2).  DIR 0: x, 1: y.
+// divergence of Sec. 2.2; Euler).  DIR 0: x, 1: y.
 template <int EQ, int DIR, bool FTZ = false, class T>
 __device__ __forceinline__ void flux_jvp(const T* q, const T* dq, const Phys<T>& ph, T* df)
 {
-    if constexpr (EQ == EQ_ADV) {
-        df[0] = (DIR == 0 ? ph.ax : ph.ay) * dq[0];
-    } else {
-        T u, v, r;
-        T p = pressure<FTZ>(q, ph.gamma, u, v, r);
-        T vn = DIR == 0 ? u : v;
-        T dvn = ((DIR == 0 ? dq[1] : dq[2]) - vn * dq[0]) * r;
-        T dp = (ph.gamma - T(1)) * (dq[3] - (u * dq[1] + v * dq[2]) + T(0.5) * (u * u + v * v) * dq[0]);
-        df[0] = DIR == 0 ? dq[1] : dq[2];
-        df[1] = dq[1] * vn + q[1] * dvn + (DIR == 0 ? dp : T(0));
-        df[2] = dq[2] * vn + q[2] * dvn + (DIR == 1 ? dp : T(0));
-        df[3] = (dq[3] + dp) * vn + (q[3] + p) * dvn;
-    }
+    static_assert(EQ == EQ_EULER, "advection kernels need no point flux");
+    T u, v, r;
+    T p = pressure<FTZ>(q, ph.gamma, u, v, r);
+    T vn = DIR == 0 ? u : v;
+    T dvn = ((DIR == 0 ? dq[1] : dq[2]) - vn * dq[0]) * r;
+    T dp = (ph.gamma - T(1)) * (dq[3] - (u * dq[1] + v * dq[2]) + T(0.5) * (u * u + v * v) * dq[0]);
+    df[0] = DIR == 0 ? dq[1] : dq[2];
+    df[1] = dq[1] * vn + q[1] * dvn + (DIR == 0 ? dp : T(0));
+    df[2] = dq[2] * vn + q[2] * dvn + (DIR == 1 ? dp : T(0));
+    df[3] = (dq[3] + dp) * vn + (q[3] + p) * dvn;
 }
 
 // |lambda| of an acoustic field with the Harten-Hyman entropy fix: lam_m,
@@ -391,16 +381,12 @@ struct Ref {
 template <int EQ, class T>
 __device__ __forceinline__ Ref<T> make_ref(const T* q, const Phys<T>& ph)
 {
+    static_assert(EQ == EQ_EULER, "the delta form is the Euler kernels' only");
     Ref<T> r;
-    constexpr int V = NVars<EQ>::value;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) r.q[k] = k < V ? q[k] : T(0);
-    if constexpr (EQ == EQ_EULER) {
-        r.p = pressure(q, ph.gamma, r.u, r.v);
-        r.H = q[3] + r.p;
-    } else {
-        r.u = r.v = r.p = r.H = T(0);
-    }
+    for (int k = 0; k < 4; ++k) r.q[k] = q[k];
+    r.p = pressure(q, ph.gamma, r.u, r.v);
+    r.H = q[3] + r.p;
     return r;
 }
 
@@ -413,34 +399,28 @@ __device__ __forceinline__ Ref<T> make_ref(const T* q, const Phys<T>& ph)
 template <int EQ, int DIR, class T>
 __device__ __forceinline__ void dflux_speed(const Ref<T>& r, const T* d, const Phys<T>& ph, T* out, T& speed)
 {
-    if constexpr (EQ == EQ_ADV) {
-        const T an = DIR == 0 ? ph.ax : ph.ay;
-        out[0] = an * d[0];
-        speed = an >= T(0) ? an : -an;
+    const T inv = frcp(r.q[0] + d[0]);
+    const T du = (d[1] - r.u * d[0]) * inv;
+    const T dv = (d[2] - r.v * d[0]) * inv;
+    const T m1 = r.q[1] + d[1], n1 = r.q[2] + d[2];
+    const T dmu = d[1] * r.u + m1 * du;
+    const T dnv = d[2] * r.v + n1 * dv;
+    const T dp = (ph.gamma - T(1)) * (d[3] - T(0.5) * (dmu + dnv));
+    const T dH = d[3] + dp;
+    const T dvn = DIR == 0 ? du : dv;
+    const T vn0 = DIR == 0 ? r.u : r.v;
+    if (DIR == 0) {
+        out[0] = d[1];
+        out[1] = dmu + dp;
+        out[2] = d[2] * r.u + n1 * du;
     } else {
-        const T inv = frcp(r.q[0] + d[0]);
-        const T du = (d[1] - r.u * d[0]) * inv;
-        const T dv = (d[2] - r.v * d[0]) * inv;
-        const T m1 = r.q[1] + d[1], n1 = r.q[2] + d[2];
-        const T dmu = d[1] * r.u + m1 * du;
-        const T dnv = d[2] * r.v + n1 * dv;
-        const T dp = (ph.gamma - T(1)) * (d[3] - T(0.5) * (dmu + dnv));
-        const T dH = d[3] + dp;
-        const T dvn = DIR == 0 ? du : dv;
-        const T vn0 = DIR == 0 ? r.u : r.v;
-        if (DIR == 0) {
-            out[0] = d[1];
-            out[1] = dmu + dp;
-            out[2] = d[2] * r.u + n1 * du;
-        } else {
-            out[0] = d[2];
-            out[1] = d[1] * r.v + m1 * dv;
-            out[2] = dnv + dp;
-        }
-        out[3] = dH * vn0 + (r.H + dH) * dvn;
-        const T vn1 = vn0 + dvn;
-        speed = (vn1 >= T(0) ? vn1 : -vn1) + fsqrt(ph.gamma * (r.p + dp) * inv);
+        out[0] = d[2];
+        out[1] = d[1] * r.v + m1 * dv;
+        out[2] = dnv + dp;
     }
+    out[3] = dH * vn0 + (r.H + dH) * dvn;
+    const T vn1 = vn0 + dvn;
+    speed = (vn1 >= T(0) ? vn1 : -vn1) + fsqrt(ph.gamma * (r.p + dp) * inv);
 }
 
 template <int EQ, int DIR, class T>
@@ -451,12 +431,12 @@ __device__ __forceinline__ void dflux(const Ref<T>& r, const T* d, const Phys<T>
 }
 
 // Common flux relative to the reference: G = F*(ref + dm, ref + dp) - f(ref),
-// Rusanov (lambda = larger one-sided speed) or upwind (advection).
+// Rusanov (lambda = larger one-sided speed) or Roe.
 template <int EQ, int FLUX, int DIR, class T>
 __device__ __forceinline__ void common_flux_delta(const Ref<T>& r, const T* dm, const T* dp, const Phys<T>& ph,
                                                   T* G)
 {
-    if constexpr (EQ == EQ_EULER && FLUX == FLUX_ROE) {
+    if constexpr (FLUX == FLUX_ROE) {
         // no difference form of Roe's flux: the flux of the full states,
         // shifted to the reference
         T qm[4], qp[4], F[4], f0[4];
@@ -470,16 +450,6 @@ __device__ __forceinline__ void common_flux_delta(const Ref<T>& r, const T* dm, 
         else flux_y<EQ>(r.q, ph, f0);
 #pragma unroll
         for (int k = 0; k < 4; ++k) G[k] = F[k] - f0[k];
-        return;
-    }
-    if constexpr (EQ == EQ_ADV) {
-        const T an = DIR == 0 ? ph.ax : ph.ay;
-        if constexpr (FLUX == FLUX_UPWIND || FLUX == FLUX_ROE) {
-            G[0] = an >= T(0) ? an * dm[0] : an * dp[0];
-        } else {
-            const T lam = an >= T(0) ? an : -an;
-            G[0] = T(0.5) * (an * dm[0] + an * dp[0]) - T(0.5) * lam * (dp[0] - dm[0]);
-        }
     } else {
         T Fm[4], Fp[4], sm, sp;
         dflux_speed<EQ, DIR>(r, dm, ph, Fm, sm);
@@ -490,102 +460,33 @@ __device__ __forceinline__ void common_flux_delta(const Ref<T>& r, const T* dm, 
     }
 }
 
-// ---- transposed linearisations (discrete adjoint) --------------------------
+// ---- transposed linearisations of advection (discrete adjoint) -------------
 
-// qbar += (dF_DIR/dq)^T w at state q (F_DIR the x- or y-flux of Eq. 4).
+// (Euler: cpr_adjoint_quad.cuh.)
+
+// qbar += (dF_DIR/dq)^T w (at any state q).
 template <int EQ, int DIR, class T>
 __device__ __forceinline__ void flux_vjp(const T* q, const T* w, const Phys<T>& ph, T* qbar)
 {
-    if constexpr (EQ == EQ_ADV) {
-        qbar[0] += (DIR == 0 ? ph.ax : ph.ay) * w[0];
-    } else {
-        const T g1 = ph.gamma - T(1);
-        const T r = q[0], ir = frcp(r);
-        const T u = q[1] * ir, v = q[2] * ir;
-        const T p = g1 * (q[3] - T(0.5) * (q[1] * u + q[2] * v));
-        const T vn = DIR == 0 ? u : v;
-        const T nx = DIR == 0 ? T(1) : T(0), ny = DIR == 0 ? T(0) : T(1);
-        const T dvn[4] = {-vn * ir, nx * ir, ny * ir, T(0)};
-        const T dpq[4] = {g1 * T(0.5) * (u * u + v * v), -g1 * u, -g1 * v, g1};
-        const T C = w[1] * q[1] + w[2] * q[2] + w[3] * (q[3] + p);
-        const T Pc = w[1] * nx + w[2] * ny + w[3] * vn;
-        qbar[0] += C * dvn[0] + Pc * dpq[0];
-        qbar[1] += w[0] * nx + vn * w[1] + C * dvn[1] + Pc * dpq[1];
-        qbar[2] += w[0] * ny + vn * w[2] + C * dvn[2] + Pc * dpq[2];
-        qbar[3] += vn * w[3] + Pc * dpq[3];
-    }
+    static_assert(EQ == EQ_ADV, "Euler: jacobian_t");
+    qbar[0] += (DIR == 0 ? ph.ax : ph.ay) * w[0];
 }
 
-// Gradient of the signal speed |Vn| + c (Euler).
-template <int DIR, class T>
-__device__ __forceinline__ void speed_grad(const T* q, const Phys<T>& ph, T* gs)
-{
-    const T g1 = ph.gamma - T(1);
-    const T r = q[0], ir = frcp(r);
-    const T u = q[1] * ir, v = q[2] * ir;
-    const T p = g1 * (q[3] - T(0.5) * (q[1] * u + q[2] * v));
-    const T cs = fsqrt(ph.gamma * p * ir);
-    const T vn = DIR == 0 ? u : v;
-    const T sg = vn >= T(0) ? T(1) : T(-1);
-    const T nx = DIR == 0 ? T(1) : T(0), ny = DIR == 0 ? T(0) : T(1);
-    const T dvn[4] = {-vn * ir, nx * ir, ny * ir, T(0)};
-    const T dpq[4] = {g1 * T(0.5) * (u * u + v * v), -g1 * u, -g1 * v, g1};
-    const T k = ph.gamma * frcp(T(2) * cs * r);
-#pragma unroll
-    for (int m = 0; m < 4; ++m) gs[m] = sg * dvn[m] + k * (dpq[m] - (m == 0 ? p * ir : T(0)));
-}
-
-// Transpose of the common flux (Rusanov with lambda the larger one-sided
-// speed, differentiated on the branch the forward takes; or upwind):
-// qbm, qbp = cotangents of the lower and upper states for cotangent w.
+// Transpose of the common flux (Rusanov or upwind): qbm, qbp = cotangents of
+// the lower and upper states for cotangent w (at any states qm, qp).
 template <int EQ, int FLUX, int DIR, class T>
 __device__ __forceinline__ void common_flux_vjp(const T* qm, const T* qp, const T* w, const Phys<T>& ph, T* qbm,
                                                 T* qbp)
 {
-    if constexpr (EQ == EQ_ADV) {
-        const T an = DIR == 0 ? ph.ax : ph.ay;
-        if constexpr (FLUX == FLUX_UPWIND) {
-            qbm[0] = an >= T(0) ? an * w[0] : T(0);
-            qbp[0] = an >= T(0) ? T(0) : an * w[0];
-        } else {
-            const T lam = an >= T(0) ? an : -an;
-            qbm[0] = T(0.5) * an * w[0] + T(0.5) * lam * w[0];
-            qbp[0] = T(0.5) * an * w[0] - T(0.5) * lam * w[0];
-        }
+    static_assert(EQ == EQ_ADV, "Euler: face_t");
+    const T an = DIR == 0 ? ph.ax : ph.ay;
+    if constexpr (FLUX == FLUX_UPWIND) {
+        qbm[0] = an >= T(0) ? an * w[0] : T(0);
+        qbp[0] = an >= T(0) ? T(0) : an * w[0];
     } else {
-        T hw[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            hw[k] = T(0.5) * w[k];
-            qbm[k] = T(0);
-            qbp[k] = T(0);
-        }
-        flux_vjp<EQ, DIR>(qm, hw, ph, qbm);
-        flux_vjp<EQ, DIR>(qp, hw, ph, qbp);
-        T um, vm, up, vp, rm, rp;
-        const T pm = pressure(qm, ph.gamma, um, vm, rm);
-        const T pp = pressure(qp, ph.gamma, up, vp, rp);
-        const T vnm = DIR == 0 ? um : vm, vnp = DIR == 0 ? up : vp;
-        const T sm = (vnm >= T(0) ? vnm : -vnm) + fsqrt(ph.gamma * pm * rm);
-        const T sp = (vnp >= T(0) ? vnp : -vnp) + fsqrt(ph.gamma * pp * rp);
-        const T lam = sm >= sp ? sm : sp;
-        T jump = T(0);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            qbm[k] += T(0.5) * lam * w[k];
-            qbp[k] -= T(0.5) * lam * w[k];
-            jump += w[k] * (qp[k] - qm[k]);
-        }
-        T gs[4];
-        if (sm >= sp) {
-            speed_grad<DIR>(qm, ph, gs);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) qbm[k] -= T(0.5) * jump * gs[k];
-        } else {
-            speed_grad<DIR>(qp, ph, gs);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) qbp[k] -= T(0.5) * jump * gs[k];
-        }
+        const T lam = an >= T(0) ? an : -an;
+        qbm[0] = T(0.5) * an * w[0] + T(0.5) * lam * w[0];
+        qbp[0] = T(0.5) * an * w[0] - T(0.5) * lam * w[0];
     }
 }
 
@@ -644,25 +545,21 @@ __device__ __forceinline__ Pr<T> prcp(Pr<T> a) { return pmk(frcp(a.v.x), frcp(a.
 template <int EQ, int DIR, class T>
 __device__ __forceinline__ void flux_pair(const Pr<T>* q, const Phys<T>& ph, Pr<T>* f)
 {
-    if constexpr (EQ == EQ_ADV) {
-        f[0] = pmul(pbc(DIR == 0 ? ph.ax : ph.ay), q[0]);
+    const Pr<T> r = prcp(q[0]);
+    const Pr<T> u = pmul(q[1], r), v = pmul(q[2], r);
+    Pr<T> t = pmul(q[1], u);
+    t = pfma(q[2], v, t);
+    const Pr<T> p = pmul(pbc(ph.gamma - T(1)), pfma(pbc(T(-0.5)), t, q[3]));
+    if constexpr (DIR == 0) {
+        f[0] = q[1];
+        f[1] = pfma(q[1], u, p);
+        f[2] = pmul(q[2], u);
+        f[3] = pmul(padd(q[3], p), u);
     } else {
-        const Pr<T> r = prcp(q[0]);
-        const Pr<T> u = pmul(q[1], r), v = pmul(q[2], r);
-        Pr<T> t = pmul(q[1], u);
-        t = pfma(q[2], v, t);
-        const Pr<T> p = pmul(pbc(ph.gamma - T(1)), pfma(pbc(T(-0.5)), t, q[3]));
-        if constexpr (DIR == 0) {
-            f[0] = q[1];
-            f[1] = pfma(q[1], u, p);
-            f[2] = pmul(q[2], u);
-            f[3] = pmul(padd(q[3], p), u);
-        } else {
-            f[0] = q[2];
-            f[1] = pmul(q[1], v);
-            f[2] = pfma(q[2], v, p);
-            f[3] = pmul(padd(q[3], p), v);
-        }
+        f[0] = q[2];
+        f[1] = pmul(q[1], v);
+        f[2] = pfma(q[2], v, p);
+        f[3] = pmul(padd(q[3], p), v);
     }
 }
 

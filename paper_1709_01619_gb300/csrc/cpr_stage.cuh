@@ -1,7 +1,9 @@
-// cpr_stage.cuh -- fused CPR residual + SSP-RK3 stage kernel.
+// cpr_stage.cuh -- the CPR residual and SSP-RK3 stages: the scheme, the stage
+// modes, what all stage kernels share, and the kernel of the stand-alone FP32
+// Euler residual.
 //
-// One CTA owns a tile of TX x TY elements and computes, for every solution
-// point of the tile, the CPR right-hand side of Sec. 2.2 (Eq. 16-17)
+// A CTA owns a tile of TX x TY elements and computes, for every solution point
+// of the tile, the CPR right-hand side of Sec. 2.2 (Eq. 16-17)
 //   R_ab = -(2/hx) [ sum_l D_al f_lb + (F*_L,b - f_L,b) g_L'(xi_a) + (F*_R,b - f_R,b) g_R'(xi_a) ]
 //          -(2/hy) [ sum_l D_bl g_al + (G*_B,a - g_B,a) g_L'(eta_b) + (G*_T,a - g_T,a) g_R'(eta_b) ]
 // and then one stage of the three-stage SSP Runge-Kutta scheme of Sec. 4, in
@@ -14,12 +16,17 @@
 //     so that the O(1e-3) update of an O(1) state does not lose its low bits
 //     every stage.  hi' goes to a second buffer (neighbour CTAs still read hi).
 //
+// Kernels: FP32 Euler stages cpr_stage_quad.cuh, FP64 Euler cpr_stage_f64.cuh,
+// advection cpr_stage_adv.cuh.  The tile below runs the stand-alone FP32 Euler
+// residual (mode 0); built with -DCPR_FP32_DELTA=1, in the delta form, every FP32
+// Euler stage.
+//
 // Thread roles (N = p+1 points per direction, NT = TX*TY*N threads): thread
 // (el, k) is the x-line "row k of element el" and the y-line "column k of
 // element el".  Its row comes from HBM into registers; its column is read
 // from the shared-memory copy of the tile.
 //
-// Delta form (FP32): every flux is evaluated as an exact algebraic difference
+// Delta form: every flux is evaluated as an exact algebraic difference
 // f(q_ref + d) - f(q_ref) from the state q_ref at point (0, 0) of its element.
 // The divergence and the edge terms only need flux differences (the rows of
 // D sum to zero, the edge weights sum to one), so the rounding error of the
@@ -27,7 +34,6 @@
 // formed relative to the upper (right/top) element's reference and shifted by
 // f(ref_upper) - f(ref_lower) for the lower element's jump; on the tile's
 // right/top edge it is formed relative to the lower element's reference.
-// FP64 evaluates the fluxes directly (reference zero).
 //
 // Phases (one barrier after each of 1-3):
 //   1 own row: into the tile copy, x-line (flux differences, d/dxi, edge
@@ -96,9 +102,7 @@ struct StageLayout {
     // The y-derivatives go over the dead tile copy in phase 3 (a buffer of
     // their own, written in phase 2, holds fewer registers across the
     // barrier but leaves too little of the SM's shared memory / L1 to L1).
-    static constexpr bool RYSEP = false;
-    static constexpr int SQ = V * E * ES;              // tile copy
-    static constexpr int RY = RYSEP ? SQ : 0;          // y-derivatives of the flux
+    static constexpr int SQ = V * E * ES;              // tile copy, then the y-derivatives
     static constexpr int XR = V * TY * (TX + 1) * N;   // right edge states, elements -1..TX-1
     static constexpr int XH = V * TY * N;              // left edge states of the right halo
     static constexpr int XF = V * E * N;               // right edge fluxes, then the right jumps
@@ -107,7 +111,7 @@ struct StageLayout {
     static constexpr int YF = V * E * N;               // top edge fluxes, then the top jumps
     static constexpr int JB = V * E * N;               // bottom jumps
     static constexpr int RF = DELTA ? V * PE : 0;      // element reference states
-    static constexpr int TOTAL = SQ + RY + XR + XH + XF + YT + YH + YF + JB + RF;
+    static constexpr int TOTAL = SQ + XR + XH + XF + YT + YH + YF + JB + RF;
     // point (b, a) (row b, column a) of element el in a tile array
     __device__ static int sq(int v, int el, int b, int a)
     {
@@ -399,20 +403,19 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, const Tab<T>& 
     constexpr int N = P + 1, NN = N * N, V = NVars<EQ>::value;
     constexpr int NT = TX * TY * N;
     // Two-lane path (pairs of points of a line; packed FP32 instructions):
-    // LP divergence, fluxes evaluated directly; even N, and N = 5 in FP32
-    // (FP64 pairs are two scalar operations, so an odd line's last pair
-    // would only add work there; for N = 3 in FP32 it measured 1 % faster on
-    // the batch and 1 % slower on the limited run).  An odd line's last pair
-    // repeats its last point (PH): the table pairs carry zero for it, and
-    // its derivative and residual lanes are not stored.
-    constexpr bool PAIRED = DIV == DIV_LP && !DELTA && (N % 2 == 0 || (sizeof(T) == 4 && N == 5));
+    // LP divergence, fluxes evaluated directly; even N, and N = 5 (for N = 3
+    // it measured 1 % faster on the batch and 1 % slower on the limited run).
+    // An odd line's last pair repeats its last point (PH): the table pairs
+    // carry zero for it, and its derivative and residual lanes are not stored.
+    static_assert(EQ == EQ_EULER && sizeof(T) == 4, "FP64 and advection have tiles of their own");
+    constexpr bool PAIRED = DIV == DIV_LP && !DELTA && (N % 2 == 0 || N == 5);
     constexpr int NP = (N + 1) / 2;
     auto PH = [](int i) { return i < N ? i : N - 1; };
     static_assert(TX * TY >= TX + TY, "every tile-edge face point needs a thread of its own");
     using L = StageLayout<N, V, TX, TY, DELTA>;
     T* sq = reinterpret_cast<T*>(smem_raw);
-    T* ryS = L::RYSEP ? sq + L::SQ : sq;  // y-derivatives (else over the dead tile copy)
-    T* xR = sq + L::SQ + L::RY;
+    T* ryS = sq;  // y-derivatives, over the dead tile copy
+    T* xR = sq + L::SQ;
     T* xH = xR + L::XR;
     T* xF = xH + L::XH;
     T* yT = xF + L::XF;
@@ -689,12 +692,6 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, const Tab<T>& 
             yT[L::yt(v, tyc + 1, txc, kc)] = eT[v];
             yF[L::ef(v, elc, kc)] = gT[v];
         }
-        if constexpr (L::RYSEP) {
-#pragma unroll
-            for (int b = 0; b < N; ++b)
-#pragma unroll
-                for (int v = 0; v < V; ++v) ryS[L::sq(v, elc, b, kc)] = ry[b][v];
-        }
     }
     __syncthreads();
 
@@ -706,7 +703,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, const Tab<T>& 
     // neighbour's (over the neighbour's edge flux in shared memory, shifted to
     // the neighbour's reference).
     T JL[V];
-    if (validc && !L::RYSEP) {
+    if (validc) {
 #pragma unroll
         for (int b = 0; b < N; ++b)
 #pragma unroll
