@@ -24,8 +24,8 @@
 // barrier (after phase 2).
 //
 // Against the general tile, us per FP64 stage on 16^2 elements, p = 1 to 4: 6.1 /
-// 9.1 / 13.3 / 12.1 -> 4.9 / 6.0 / 6.5 / 7.6, 96^2 6.2 / 9.3 / 13.5 / 19.3 -> 5.0 /
-// 7.4 / 10.0 / 14.2; FP32 is bound by the launch (3.2 to 3.7 -> 3.1 to 3.6).
+// 9.1 / 13.3 / 12.1 -> 4.7 / 5.5 / 6.3 / 7.3, 96^2 6.2 / 9.3 / 13.5 / 19.3 -> 4.9 /
+// 7.3 / 9.8 / 13.8; FP32 is bound by the launch (3.2 to 3.7 -> 3.1 to 3.6).
 #pragma once
 
 #include "cpr_stage_quad.cuh"

@@ -17,8 +17,9 @@
 //     operations of a thread that owns a row and a column.  A grid that
 //     leaves schedulers idle runs in half the time, and a large one fills the
 //     last round of warps better.
-// 128^2 p = 3, 12 steps: 4.49 -> 3.09 ms (86 us per stage, 82 % of the FP64
-// pipe's cycles on the busiest SM); 16^2 elements, us per stage, p = 1 to 4: 25 /
+// 128^2 p = 3, 12 steps: 4.49 -> 3.09 ms (86 us per stage; the busiest scheduler
+// gets 8 of 4096 warps where 6.7 is the mean, and its FP64 pipe is busy 84 % of
+// the launch, the rest are the barriers of a tile); 16^2 elements, us per stage, p = 1 to 4: 25 /
 // 41 / 36 / 56 -> 11 / 15 / 17 / 20.  With one thread for a row and a column, the
 // same operations took 18 / 22 / 26 / 32.
 //

@@ -11,7 +11,7 @@
 // Against the same phases with one word per variable (thread instructions per
 // thread of the first increment stage: p = 2 1185 -> 695, p = 3 1080 -> 848,
 // p = 4 1450 -> 961), per pass, and with the later changes noted below: 1024^2
-// p = 3 5.27 -> 4.51 -> 4.40 ms (8 steps), 1365 x 1363 p = 2 5.67 -> 4.70 -> 4.63
+// p = 3 5.27 -> 4.51 -> 4.32 ms (8 steps), 1365 x 1363 p = 2 5.67 -> 4.70 -> 4.58
 // ms (6 steps), 821 x 819 p = 4 5.64 -> 5.03 -> 4.91 ms (6 steps), 128^2 p = 3
 // 1.34 -> 1.11 -> 1.07 ms (64 steps, L2-resident).  Bound: at 1024^2 HBM in the
 // second and third stage (5.2 TB/s moved); for odd N the L1 / shared-memory data
