@@ -545,8 +545,8 @@ __device__ __forceinline__ void stage_tile_quad(const StageArgs<float>& A, const
         if (mode == MODE_INC1) {
         } else if (mode <= MODE_SO3) {
             // q1 = q + dt R, then q + c ((q_i - q) + dt R), c = 1/4, 2/3: one
-            // rounding of the state's size (the difference is exact), and
-            // weights that sum to one, where 1/3 and 2/3 in FP32 exceed it by
+            // rounding of the state's size (the difference is exact within a
+            // factor of two), and weights that sum to one, where 1/3 and 2/3 in FP32 exceed it by
             // 3e-8, a growth of every step (limited runs of 8 steps, error
             // against 64 bits over twelve states: p = 1 1.15e-7 -> 4.9e-8, p = 2
             // 1.14e-7 -> 5.8e-8, p = 3 1.09e-7 -> 7.7e-8)
